@@ -189,15 +189,16 @@ int slots_for(int n, int mode, const int8_t *by_n = nullptr, int dflt = 2)
     return n >= v ? v : std::min(n, 2);  // a layout wider than the race falls back
 }
 
-// A run of work items of one race, each of `chunk` rollouts, the first from rollout k0 on;
-// `first` is the run's first index in the list (the run ends where the next one starts).
+// A run of work items of one race, each of `chunk` rollouts, the first from rollout k0 on (tickets:
+// all of them from k0); `first` is the run's first index in the list (the run ends where the next
+// one starts).
 struct ItemRun {
     int32_t race, k0, chunk, first;
 };
 
 // items[i] for every list index i: the run holding i (the last whose first index is at most i,
 // by binary search over the runs in list order), then its item i - first.
-__global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, int32_t total,
+__global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, int32_t total, bool tickets,
                              bbe::WorkItem *__restrict__ items)
 {
     const int32_t i = int32_t(blockIdx.x * blockDim.x + threadIdx.x);
@@ -209,7 +210,7 @@ __global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, i
         else hi = mid - 1;
     }
     const ItemRun r = runs[lo];
-    items[i] = bbe::WorkItem{r.race, r.k0 + (i - r.first) * r.chunk, r.chunk, 0};
+    items[i] = bbe::WorkItem{r.race, tickets ? r.k0 : r.k0 + (i - r.first) * r.chunk, r.chunk, 0};
 }
 
 bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
@@ -271,6 +272,11 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
         }
         if (b->seg_cap == 0) race_items = kMaxItemsPerRace;
     }
+    b->per_lane = int32_t(per_lane);
+    b->tickets = b->default_slots == 2;
+    // at least four turns for each warp that is resident (28 per SM): an item too long leaves the
+    // others waiting at the end
+    b->most = int32_t(std::min<int64_t>(INT32_MAX, std::max<int64_t>(1, total_rollouts / (int64_t(std::max(1, b->num_sms)) * 28 * 4))));
     size_t total = 0;
     for (int r = 0; r < b->n_races; ++r) {
         const int n = b->h_off[r + 1] - b->h_off[r];
@@ -305,7 +311,8 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
         std::stable_sort(pg.begin(), pg.end(), [](const RacePlan &x, const RacePlan &y) { return x.cost_rem > y.cost_rem; });
         for (const RacePlan &pl : pg) {
             if (pl.rem == 0) continue;
-            runs.push_back(ItemRun{pl.race, int32_t(pl.k0 + pl.full * pl.chunk), int32_t(pl.rem), listed});
+            if (b->tickets) runs.push_back(ItemRun{pl.race, int32_t(pl.k0), int32_t(pl.chunk), listed});
+            else runs.push_back(ItemRun{pl.race, int32_t(pl.k0 + pl.full * pl.chunk), int32_t(pl.rem), listed});
             listed += 1;
         }
         b->n_items_v[g] = listed - before;
@@ -324,7 +331,7 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
     if (!runs.empty()) {
         BBE_CUDA_TRY(pool_alloc(reinterpret_cast<void **>(&d_runs), runs.size() * sizeof(ItemRun), upload));
         BBE_CUDA_TRY(cudaMemcpyAsync(d_runs, runs.data(), runs.size() * sizeof(ItemRun), cudaMemcpyHostToDevice, upload));
-        expand_items<<<unsigned((listed + 255) / 256), 256, 0, upload>>>(d_runs, int32_t(runs.size()), listed, fresh);
+        expand_items<<<unsigned((listed + 255) / 256), 256, 0, upload>>>(d_runs, int32_t(runs.size()), listed, b->tickets, fresh);
         BBE_CUDA_TRY(cudaGetLastError());
         BBE_CUDA_TRY(cudaFreeAsync(d_runs, upload));
     }
@@ -355,6 +362,10 @@ bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *ste
     l.items = b->d_items + first;
     l.n_items = b->n_items_v[g];
     l.queue = b->d_queue + g;
+    l.next = b->tickets ? b->d_next : nullptr;
+    l.per_lane = b->per_lane;
+    l.most = b->most;
+    l.contenders = b->tickets ? 1 : 0;
     l.counts = counts;
     l.steps = reinterpret_cast<unsigned long long *>(steps);
     l.status = b->d_status;
@@ -369,14 +380,19 @@ bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *ste
     return l;
 }
 
+// Queue heads, status and, behind them, the races' ticket counters: one range.
+cudaError_t reset_queue(const bbe_batch *b, cudaStream_t s)
+{
+    return cudaMemsetAsync(b->d_queue, 0, (kGroups + 1 + (b->tickets ? size_t(b->n_races) : 0)) * sizeof(int32_t), s);
+}
+
 // The launch sequence of one rollout pass: reset queues, status and outputs, then one
 // persistent kernel per non-empty slots-per-lane group, the group with most slots first.
 // With a side stream the first kernel runs on `s` and the others on `side`, so that they
 // fill SMs as the first kernel's blocks retire.
 cudaError_t enqueue_pass(const bbe_batch *b, int32_t *counts, int64_t *steps, cudaStream_t s, cudaStream_t side)
 {
-    cudaError_t e = cudaMemsetAsync(b->d_queue, 0, kGroups * sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_status, 0, sizeof(int32_t), s);
+    cudaError_t e = reset_queue(b, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, size_t(b->n_total) * sizeof(int32_t), s);
     if (e == cudaSuccess && steps) e = cudaMemsetAsync(steps, 0, size_t(b->n_races) * sizeof(int64_t), s);
     int groups[kGroups], ng = 0;
@@ -591,7 +607,7 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
     auto add = [&](size_t n) { bytes += (n + 255) / 256 * 256; };
     add((n_races + 1) * 4); add(n_races * 4); add(n_races * 8); add(size_t(nt) * 4); add(n_races * 4);
     for (int i = 0; i < 7; ++i) add(size_t(nt) * 4);
-    add(4 * kGroups); add(4);
+    add((kGroups + 1 + size_t(n_races)) * 4);
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e == cudaSuccess) e = pool_alloc(&b->arena, bytes, s);
@@ -608,8 +624,9 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
     float *d_d0 = carve<float>(p, nt), *d_mu = carve<float>(p, nt), *d_sigma = carve<float>(p, nt);
     float *d_rho = carve<float>(p, nt), *d_P = carve<float>(p, nt), *d_theta = carve<float>(p, nt);
     float *d_prev = carve<float>(p, nt);
-    b->d_queue = carve<int32_t>(p, kGroups);
-    b->d_status = carve<int32_t>(p, 1);
+    b->d_queue = carve<int32_t>(p, kGroups + 1 + size_t(n_races));
+    b->d_status = b->d_queue + kGroups;
+    b->d_next = b->d_status + 1;
     // A small batch's arena is assembled on the host in its own layout and goes up in one copy
     // (one transfer's overhead instead of one per array); a large one goes up array by array,
     // with no extra host pass over it.  The queue heads and status are reset before use.
@@ -744,8 +761,7 @@ bbe_status run_place_mode(bbe_batch *b, int32_t places, int32_t *place_counts, i
     if (place_counts)
         BBE_CUDA_TRY(cudaMemsetAsync(place_counts, 0, size_t(b->n_total) * size_t(places) * sizeof(int32_t), s));
     if (steps_total) BBE_CUDA_TRY(cudaMemsetAsync(steps_total, 0, size_t(b->n_races) * sizeof(int64_t), s));
-    BBE_CUDA_TRY(cudaMemsetAsync(b->d_queue, 0, kGroups * sizeof(int32_t), s));
-    BBE_CUDA_TRY(cudaMemsetAsync(b->d_status, 0, sizeof(int32_t), s));
+    BBE_CUDA_TRY(reset_queue(b, s));
     for (int g = kGroups - 1; g >= 0; --g) {
         if (b->n_items_v[g] == 0) continue;
         bbe::RolloutLaunch l = make_launch(b, place_counts, steps_total, g);

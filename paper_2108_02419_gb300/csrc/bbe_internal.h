@@ -44,8 +44,9 @@ __device__ __forceinline__ float responsiveness(float kr, float d, float invL, f
     }
 }
 
-// A unit of the persistent kernel's work queue: rollouts k_begin .. k_begin+k_count-1
-// of one race.
+// A unit of the persistent kernel's work queue: rollouts k_begin .. k_begin+k_count-1 of one race;
+// in a launch with `next` a ticket for k_count or more of the race's rollouts k_begin, .. (all its
+// tickets alike), of which the warp takes as many as its segments can share.
 struct WorkItem {
     int32_t race;
     int32_t k_begin;
@@ -58,6 +59,10 @@ struct RolloutLaunch {
     const WorkItem *items;
     int32_t n_items;
     int32_t *queue;           // work-queue head, zeroed before each launch
+    int32_t *next;            // [n_races] tickets' worth of rollouts taken, zeroed before each launch; null: none
+    int32_t per_lane;         // with next: rollouts per segment that a warp takes at a time, ..
+    int32_t most;             // .. and in all, unless one ticket is worth more
+    int32_t contenders;       // win counts: advance only the competitors that can matter (contender_line)
     int32_t *counts;          // [n_total]
     unsigned long long *steps;  // [n_races] or null
     int32_t *status;          // device status bits
@@ -189,12 +194,16 @@ struct bbe_batch {
     WorkItem *d_items = nullptr;  // items grouped by slots per lane (1, 2, 3, 4)
     int32_t n_items_v[4] = {0, 0, 0, 0};  // item counts per group
     int32_t *d_queue = nullptr;        // one queue head per group
-    int32_t *d_status = nullptr;
+    int32_t *d_status = nullptr;       // after the queue heads
+    int32_t *d_next = nullptr;         // [n_races] rollouts taken (WorkItem), after the status
 
     bbe_launch_cfg cfg{};
     int8_t slots_by_n[BBE_MAX_COMPETITORS + 1] = {};  // layout per competitor count (0: the default)
     int8_t default_slots = 2;  // the automatic layout: two per lane, one for a batch too small to fill the GPU
     int32_t seg_cap = 0;       // segments per warp at most (0: as many as fit); set for very small batches
+    int32_t per_lane = 1;      // rollouts per segment of an item (cfg.rollouts_per_lane or less)
+    int32_t most = 1;          // rollouts that a warp takes at a time at most
+    bool tickets = false;      // the items are tickets (see WorkItem): all but very small batches
     int32_t resident[4] = {1, 1, 1, 1};  // rollout-kernel blocks resident per SM, per group
     cudaStream_t side_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;

@@ -274,6 +274,7 @@ extern "C" BBE_API bbe_status bbe_rollout_noalloc(int32_t n_races, int32_t n_com
         l.steps = reinterpret_cast<unsigned long long *>(steps_total);
         l.status = &sc->h.status;
         l.max_steps = BBE_MAX_STEPS_DEFAULT;
+        l.contenders = 1;
         l.block = block;
         l.grid = sms * std::max(1, std::min(16, bbe::rollout_resident_blocks(int(dist), kSlots, block)));
         l.grid = std::max(1, std::min(l.grid, (l.n_items + block / 32 - 1) / (block / 32)));  // no idle warps

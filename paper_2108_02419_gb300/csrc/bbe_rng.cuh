@@ -48,6 +48,58 @@ __device__ __forceinline__ Words4 philox4x32_10(uint32_t c0, uint32_t c1, uint32
     return Words4{c0, c1, c2, c3};
 }
 
+// The rollout kernel's counters (k, block, c, r) differ from block to block of a rollout in the
+// second word only, so of the first four rounds just what follows from that word is left to do for a
+// block (8 of 40 multiplies fewer); StreamWords holds the rest, computed once per rollout.  The
+// words are the same as philox4x32_10's.
+struct StreamWords {
+    uint32_t a, d, e, f, g;
+};
+
+__device__ __forceinline__ StreamWords stream_words(uint32_t k, uint32_t c, uint32_t r, const uint32_t (&rk)[20])
+{
+    StreamWords s;
+    // round 1: c0 = a ^ block, c1 = lo1, c2 = b, c3 = lo0
+    const uint32_t lo0 = 0xD2511F53u * k, lo1 = 0xCD9E8D57u * c;
+    const uint32_t b = __umulhi(0xD2511F53u, k) ^ r ^ rk[1];
+    s.a = __umulhi(0xCD9E8D57u, c) ^ rk[0];
+    // round 2: c0 = c02, c2 = hi(M0 c0) ^ d
+    const uint32_t c02 = __umulhi(0xCD9E8D57u, b) ^ lo1 ^ rk[2];
+    s.d = lo0 ^ rk[3];
+    // round 3: c0 = hi(M1 c2) ^ e, c2 = f ^ lo(M0 c0 of round 2), c3 = lo(M0 c02)
+    s.e = 0xCD9E8D57u * b ^ rk[4];
+    s.f = __umulhi(0xD2511F53u, c02) ^ rk[5];
+    // round 4: c2 = hi(M0 c0) ^ g
+    s.g = 0xD2511F53u * c02 ^ rk[7];
+    return s;
+}
+
+__device__ __forceinline__ Words4 philox4x32_10_from(const StreamWords &s, uint32_t blk, const uint32_t (&rk)[20])
+{
+    uint32_t c0 = s.a ^ blk;  // round 1
+    const uint32_t hi2 = __umulhi(0xD2511F53u, c0), lo2 = 0xD2511F53u * c0;
+    uint32_t c2 = hi2 ^ s.d;  // round 2
+    uint32_t c1 = 0xCD9E8D57u * c2;
+    c0 = __umulhi(0xCD9E8D57u, c2) ^ s.e;  // round 3
+    c2 = s.f ^ lo2;
+    const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
+    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
+    c0 = hi1 ^ c1 ^ rk[6];  // round 4
+    c2 = hi0 ^ s.g;
+    c1 = lo1;
+    uint32_t c3 = lo0;
+#pragma unroll
+    for (int i = 4; i < 10; ++i) {
+        const uint32_t h0 = __umulhi(0xD2511F53u, c0), l0 = 0xD2511F53u * c0;
+        const uint32_t h1 = __umulhi(0xCD9E8D57u, c2), l1 = 0xCD9E8D57u * c2;
+        c0 = h1 ^ c1 ^ rk[2 * i];
+        c2 = h0 ^ c3 ^ rk[2 * i + 1];
+        c1 = l1;
+        c3 = l0;
+    }
+    return Words4{c0, c1, c2, c3};
+}
+
 // The float arithmetic below works on two values at once (__ffma2_rn, __fadd2_rn, __fmul2_rn:
 // one instruction for both, each component rounded exactly as __fmaf_rn, __fadd_rn and
 // __fmul_rn round it), because a Philox block always feeds two Box-Muller pairs.

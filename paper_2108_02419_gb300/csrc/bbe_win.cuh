@@ -14,15 +14,19 @@
 // position, then index), whose address it keeps in a register.  In a segment where every
 // successor is strictly in front, the successor is i+.  The same read detects an overtake or
 // an equal position (successor not strictly in front); on that rare step the segment is
-// re-sorted by odd-even transposition over a rank table in shared memory, and a slot whose
-// successor stands level with it takes the first later rank strictly in front.
+// re-ranked, and a slot whose successor stands level with it takes the first later rank strictly
+// in front.
 //
-// The step loop is unrolled over the four steps of a Philox block: a block draws one
-// Philox4x32-10 output per slot and both of its Box-Muller pairs, then runs four steps whose
-// normals are registers chosen at compile time.  Every rollout starts on a block boundary (a
+// The step loop goes by the four steps of a Philox block: a block draws one Philox4x32-10 output
+// per slot (from words kept per rollout, StreamWords) and both of its Box-Muller pairs, then runs
+// four steps whose normals are registers chosen at compile time.  Every rollout starts on a block boundary (a
 // segment that finishes waits for the next one; the counter of step t is t >> 2 in any case).
 // A finished segment takes its next rollout index from a per-warp counter, so the segments of
 // a work item stay busy until its rollouts run out.
+//
+// Who is advanced.  For win counts only the competitors that can matter to the first finish are
+// (contender_line); they take the slots, so a warp has room for more segments.  A work item is a
+// ticket for some of a race's rollouts, and the warp takes as many as its segments can share.
 //
 // Finishing.  A ballot finds the steps with finishers; each finisher offers the key
 // (within-step crossing time tau = (L - d) / S, slot) to its segment's minimum in shared
@@ -55,6 +59,7 @@ namespace win {
 
 constexpr unsigned kAll = 0xffffffffu;
 constexpr unsigned long long kNoKey = ~0ull;
+constexpr uint8_t kNoSub = 255;
 
 template <int V>
 struct WinStage {
@@ -64,23 +69,124 @@ struct WinStage {
     float4 pq[32];                      // per competitor: (mu, sigma, P, theta)
     float kr[32];                       // per competitor: kappa (2 rho - 1)
     float d0[32], prev0[32];            // per competitor: start state of every rollout
-    int rank0[32], byrank0[32];         // start rank of competitor c; competitor at start rank r
-    int wins[32];                       // wins per competitor in the current work item
-    int order[NS];                      // order[segment base + r]: slot holding rank r
-    int rnk[NS];                        // rank of each slot
-    int flag[NS];                       // by segment base + rank: the slot there swaps with its successor
+    uint4 ph[NS];                       // per slot: the current rollout's Philox constants (StreamWords)
+    unsigned pha[NS];
     unsigned segk[NS];                  // by segment base: rollout index handed to a restart
+    int wins[32];                       // wins per competitor in the current work item
     unsigned long long key[NS];         // by segment base: least crossing key of the block (win mode)
-    unsigned long long fkey[NS];        // place mode: each slot's crossing (sub-step, slot) of the block, or none
-    float2 fcross[NS];                  // place mode: (d, S) of that crossing step
+    float2 fcross[NS];                  // place mode: (d, S) of each slot's crossing in the block
+    // Rank order (ascending position, then slot).  A segment of n slots has n + 1 entries of `order`,
+    // the slots by rank and the sentinel behind them, so the entry after a slot's own is its
+    // successor's; `at` is a slot's own entry and `flag` marks the entries that swap with the next.
+    uint8_t order[2 * NS + 4], flag[2 * NS + 4];
+    uint8_t at[NS];
+    uint8_t fsub[NS];                   // place mode: sub-step of each slot's crossing in the block, or kNoSub
+    uint8_t base[NS], rbase[NS];        // first slot and first order entry of each slot's segment
+    uint8_t rank0[32], byrank0[32];     // start rank of competitor c; competitor at start rank r
+    uint8_t comp[32];                   // the race's index of competitor c (its stream and its count)
     unsigned next_k;                    // next rollout index of the work item
 };
 
-template <int DIST>
-__device__ __forceinline__ void draw_block(uint32_t k, uint32_t blk, uint32_t c, uint32_t rid,
-                                           const uint32_t (&rkey)[20], float (&z)[4])
+__device__ __forceinline__ float warp_min(float v)
 {
-    const Words4 wd = philox4x32_10(k, blk, c, rid, rkey);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(kAll, v, o));
+    return v;
+}
+
+__device__ __forceinline__ float warp_max(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kAll, v, o));
+    return v;
+}
+
+// The contenders of a race.  A first finisher is decided among the competitors near the front, and
+// Eq. 1 passes influence from front to back only, so a competitor that is certain to stay short of
+// the line until a rollout ends cannot change who wins it, nor when.  contender_line returns a
+// position such that, in every rollout that ends within H steps (H is set here), the competitors
+// behind it have no effect on the first finisher: a rollout of the others alone, each on its own
+// stream, has the same winner and the same number of steps.  -inf: nobody is ruled out.
+//
+// The bound, for any draws.  A free step is at most F = max R P (mu + z_max sigma) (the generator's
+// |z| is bounded: u1 >= 2^-24 gives a radius of at most 5.7681; sqrt(3) and 1 for the other two
+// distributions) and at least the previous steps given.  A blocked step is R min(own previous step, that
+// of the competitor in front), so it exceeds F only for a competitor whose R can exceed 1 (the set
+// D; lambda is the largest R), and then
+//   S_c(t) > lambda^k F  =>  S(t-1) > lambda^(k-1) F for c and for the one in front of it, within theta.
+// Of the competitors in a stretch of track with S(t) > lambda^k F the foremost has one in front that is
+// not among them, so each level down has one member more: S_c(t) > lambda^k F takes k + 1 members of D
+// close together, whose start positions span at most G(t) + k theta, where G(t) bounds what anyone
+// covers in t steps.  With w_k the least span of k + 1 members of D at the start,
+//   G(t+1) = G(t) + F lambda^#{k : w_k <= G(t) + n theta}
+// bounds everyone's advance.  A competitor starting behind L - G(H) is short of the line for H steps; so
+// is one that gets affected by it (it was passed, so it was behind it at that time, and G(t) bounds it
+// from there on); so whoever crosses first within H steps was never behind any of them.  Rounding is
+// covered by the factors and the margin below.
+//
+// H is an estimate of the first finish with a margin of five standard deviations; a rollout that
+// is still running after H steps makes the warp redo its work item with a longer H, then with everybody.
+// x: n floats of scratch.  Called by the whole warp; lane c < n holds competitor c.
+template <int DIST, int LAW>
+__device__ __forceinline__ float contender_line(float *x, int n, int lane, float d, float mu, float sigma, float P,
+                                                float kr, float prev, float theta, float L, float t0, float invT,
+                                                float stretch, int &H)
+{
+    const bool on = lane < n;
+    constexpr float zmax = DIST == BBE_DIST_NORMAL ? 5.769f : (DIST == BBE_DIST_UNIFORM ? 1.7321f : 1.0f);
+    // expected finish at the R of the middle of the way, and the horizon
+    float T = (L - d) / (mu * P);
+    T /= 1.0f + (LAW == BBE_LAW_TIME ? kr * (fminf((t0 + 0.5f * T) * invT, 1.0f) - 0.5f) : 0.5f * kr * d / L);
+    const float h = warp_min(on ? stretch * (1.03f * T + 5.0f * sigma * sqrtf(T) / mu + 3.0f) : INFINITY);
+    if (!(h < 1e6f)) return -INFINITY;
+    H = int(h) + 1;
+    // the largest R of each competitor (linear in the position or the time: at an end of its range)
+    float R;
+    if (LAW == BBE_LAW_TIME) {
+        const float u0 = fminf(t0 * invT, 1.0f), u1 = fminf((t0 + float(H)) * invT, 1.0f);
+        R = 1.0f + fmaxf(kr * (u0 - 0.5f), kr * (u1 - 0.5f));
+    } else {
+        R = 1.0f + fmaxf(kr * (d / L - 0.5f), 0.5f * kr);
+    }
+    R *= 1.00001f;
+    const float F = 1.0001f * fmaxf(warp_max(on ? fmaxf(prev, R * P * (mu + zmax * sigma)) : 0.0f), kStepFloor);
+    const float dmin = warp_min(on ? d : INFINITY);
+    if (!(L - float(H) * F > dmin)) return -INFINITY;  // not even at the free pace
+    const float lambda = fmaxf(warp_max(on ? R : 0.0f), 1.0f);
+    const float margin = 1e-4f * L + float(n) * warp_max(on ? theta : 0.0f);
+    const bool grows = on && R > 0.9999f;
+    const unsigned D = __ballot_sync(kAll, grows);
+    const int m = __popc(D);
+    int rank = 0;
+    for (int i = 0; i < n; ++i) {
+        const float di = __shfl_sync(kAll, d, i);
+        rank += ((D >> i) & 1u) && (di < d || (di == d && i < lane)) ? 1 : 0;
+    }
+    if (grows) x[rank] = d;
+    __syncwarp();
+    float w = INFINITY;  // least span of lane + 1 members of D
+    for (int i = 0; i + lane < m; ++i) w = fminf(w, x[i + lane] - x[i]);
+    __syncwarp();
+    float G = 0.0f;
+    for (int t = 0; t < H;) {
+        const int k = __popc(__ballot_sync(kAll, w <= G + margin));
+        const float V = 1.0001f * F * powf(lambda, float(k));
+        const float next = __shfl_sync(kAll, w, k & 31);
+        int steps = H - t;
+        if (k < m) steps = min(steps, int(fminf((next - margin - G) / V, 1e6f)) + 1);
+        steps = max(steps, 1);
+        G += float(steps) * V;
+        t += steps;
+        if (!(L - G > dmin)) return -INFINITY;
+    }
+    return L - 1.001f * G - margin;
+}
+
+template <int DIST>
+__device__ __forceinline__ void draw_block(const uint4 &q, uint32_t a, uint32_t blk, const uint32_t (&rkey)[20],
+                                           float (&z)[4])
+{
+    const Words4 wd = philox4x32_10_from(StreamWords{a, q.x, q.y, q.z, q.w}, blk, rkey);
     if (DIST == BBE_DIST_NORMAL) {
         box_muller2(wd, z[0], z[1], z[2], z[3]);
     } else if (DIST == BBE_DIST_UNIFORM) {
@@ -96,12 +202,13 @@ __device__ __forceinline__ void draw_block(uint32_t k, uint32_t blk, uint32_t c,
     }
 }
 
-// Registers per thread: enough for one or two slots per lane to run without spilling at 7 or 8
-// resident 4-warp blocks per SM (measured faster than the compiler's unbounded choice), and
-// for the register-lean three- and four-slot variants.
+// Registers per thread.  Win counts: 80 for two slots per lane (6 resident 4-warp blocks per SM) and
+// 56 for one; with 72 and 48 (7 and 10 blocks) a pass over 4096 races of 20 takes 57.1 instead of
+// 54.7 ms and one small race 59 instead of 56 us.  Place mode spills nothing at 72, and fewer warps
+// cost it 1 %.  Three and four slots per lane read their parameters from shared memory.
 template <int V, int MODE>
 struct WinRegs {
-    static constexpr int value = MODE == 0 ? (V == 1 ? 48 : (V == 2 ? 72 : 80)) : (V == 1 ? 48 : (V == 2 ? 72 : 80));
+    static constexpr int value = V == 1 ? (MODE == 0 ? 56 : 48) : (V == 2 ? (MODE == 0 ? 80 : 72) : 80);
 };
 // Parameters read from shared memory each step instead of held in registers.
 template <int V>
@@ -127,13 +234,14 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
     // place mode, per warp after all the stages: the finisher of each place (by segment base +
     // place), the places filled and the sub-step of the K-th place (by segment base), then the
     // work item's [competitor][place] table
-    int *pl_ord = nullptr, *pl_n = nullptr, *pl_kj = nullptr, *pl_cnt = nullptr;
+    uint8_t *pl_ord = nullptr, *pl_n = nullptr, *pl_kj = nullptr;
+    int *pl_cnt = nullptr;
     if constexpr (MODE == 1) {
-        pl_ord = reinterpret_cast<int *>(win_smem + (blockDim.x >> 5) * sizeof(Stage)) +
-                 (threadIdx.x >> 5) * (3 * NS + l.place_cells);
+        pl_cnt = reinterpret_cast<int *>(win_smem + (blockDim.x >> 5) * sizeof(Stage)) +
+                 (threadIdx.x >> 5) * (3 * NS / 4 + l.place_cells);
+        pl_ord = reinterpret_cast<uint8_t *>(pl_cnt + l.place_cells);
         pl_n = pl_ord + NS;
         pl_kj = pl_ord + 2 * NS;
-        pl_cnt = pl_ord + 3 * NS;
     }
     const DevBatch &b = l.b;
     const int lane = threadIdx.x & 31;
@@ -141,7 +249,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         st.pos[0][NS] = make_float2(INFINITY, INFINITY);
         st.pos[1][NS] = make_float2(INFINITY, INFINITY);
     }
-    bool hit_limit = false;
     for (;;) {
         int it = 0;
         if (lane == 0) it = atomicAdd(l.queue, 1);
@@ -150,62 +257,133 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         const WorkItem w = l.items[it];
         const int r = BBE_INDEX(w.race, b.n_races, l.status);
         const int off = b.race_off[r];
-        const int n = BBE_INDEX(b.race_off[r + 1] - off - 1, 32, l.status) + 1;  // 1..32
-        (void)BBE_INDEX(off + n - 1, b.n_total, l.status);
-        const int nseg = l.seg_cap > 0 ? min(NS / n, l.seg_cap) : NS / n;  // segments of this warp
-
-        // stage the race: lane j < n loads competitor j (coalesced) and ranks it by (d0, j)
+        const int n_race = BBE_INDEX(b.race_off[r + 1] - off - 1, 32, l.status) + 1;  // 1..32
+        (void)BBE_INDEX(off + n_race - 1, b.n_total, l.status);
+        const float L = b.L[r];
+        const float invL = __fdiv_rn(1.0f, L);
+        const float t0r = LAW == BBE_LAW_TIME ? b.t0[r] : 0.0f;     // time law: elapsed steps
+        const float invTr = LAW == BBE_LAW_TIME ? b.invT[r] : 0.0f;  // time law: 1 / expected duration
+        // a ticket: nothing to do once the race's rollouts have all been taken
+        const int64_t Rr = b.R[r];
+        if (l.next != nullptr) {
+            int taken = 0;
+            if (lane == 0) taken = *reinterpret_cast<volatile int *>(l.next + r);
+            taken = __shfl_sync(kAll, taken, 0);
+            if (int64_t(taken) * w.k_count >= Rr) continue;
+        }
+        unsigned k_begin = unsigned(w.k_begin), k_count = unsigned(w.k_count);
+        // win counts: first with the contenders alone, and again only if a rollout ran past
+        // the horizon that they were chosen for
+        for (int attempt = 0;; ++attempt) {
         __syncwarp();
-        float my_d0 = INFINITY;
-        if (lane < n) {
+        // stage the race: lane j < n_race loads competitor j (coalesced)
+        float my_d0 = INFINITY, my_mu = 1.0f, my_sg = 0.0f, my_P = 1.0f, my_th = 0.0f, my_kr = 0.0f, my_pv = 0.0f;
+        if (lane < n_race) {
             const int ci = off + lane;
-            const float mu = b.mu[ci], P = b.P[ci];
+            my_mu = b.mu[ci];
+            my_P = b.P[ci];
+            my_sg = b.sigma[ci];
+            my_th = b.theta[ci];
             my_d0 = b.d0[ci];
-            st.pq[lane] = make_float4(mu, b.sigma[ci], P, b.theta[ci]);
-            st.kr[lane] = __fmul_rn(kKappa, __fsub_rn(__fmul_rn(2.0f, b.rho[ci]), 1.0f));
-            st.d0[lane] = my_d0;
-            st.prev0[lane] = b.prev0 ? b.prev0[ci] : __fmul_rn(mu, P);
-            st.wins[lane] = 0;
+            my_kr = __fmul_rn(kKappa, __fsub_rn(__fmul_rn(2.0f, b.rho[ci]), 1.0f));
+            my_pv = b.prev0 ? b.prev0[ci] : __fmul_rn(my_mu, my_P);
         }
-        int rank = 0;
-        for (int i = 0; i < n; ++i) {
+        // the n competitors advanced, in the race's order: all of them, or the contenders where
+        // that makes room for more segments
+        unsigned keep = kAll >> (32 - n_race);
+        int limit = l.max_steps;  // a rollout that reaches it ends undecided
+        if constexpr (MODE == 0) {
+            if (l.contenders && attempt < 2 && n_race > 1) {
+                int H = 0;
+                const float line = contender_line<DIST, LAW>(reinterpret_cast<float *>(posb), n_race, lane, my_d0, my_mu, my_sg,
+                                                            my_P, my_kr, my_pv, my_th, L, t0r, invTr,
+                                                            attempt == 0 ? 1.0f : 1.4f, H);
+                const unsigned front = __ballot_sync(kAll, lane < n_race && my_d0 >= line);
+                const int nf = __popc(front);
+                if (nf > 0 && (l.seg_cap > 0 ? min(NS / nf, l.seg_cap) > min(NS / n_race, l.seg_cap) : NS / nf > NS / n_race)) {
+                    keep = front;
+                    limit = min(limit, H);
+                }
+            }
+        }
+        const int n = __popc(keep);
+        const int nseg = l.seg_cap > 0 ? min(NS / n, l.seg_cap) : NS / n;  // segments of this warp
+        if (l.next != nullptr && attempt == 0) {
+            // as many rollouts as give every segment its share, in multiples of the ticket's
+            const int mult = MODE == 0 ? max(1, min(l.per_lane * nseg, l.most) / w.k_count) : 1;
+            int first = 0;
+            if (lane == 0) first = atomicAdd(l.next + r, mult);
+            const int64_t k = int64_t(__shfl_sync(kAll, first, 0)) * w.k_count;
+            if (k >= Rr) break;
+            k_begin += unsigned(k);
+            const int64_t share = int64_t(mult) * w.k_count;
+            k_count = unsigned(share < Rr - k ? share : Rr - k);
+        }
+        bool redo = false;  // a rollout of the contenders ran past their horizon
+        const bool kept = (keep >> lane) & 1u;
+        int rank = 0;  // by (d0, index)
+        for (int i = 0; i < n_race; ++i) {
             const float di = __shfl_sync(kAll, my_d0, i);
-            rank += (di < my_d0 || (di == my_d0 && i < lane)) ? 1 : 0;
+            rank += ((keep >> i) & 1u) && (di < my_d0 || (di == my_d0 && i < lane)) ? 1 : 0;
         }
-        if (lane < n) {
-            st.rank0[lane] = rank;
-            st.byrank0[BBE_INDEX(rank, 32, l.status)] = lane;
+        __syncwarp();
+        if (kept) {
+            const int c = __popc(keep & ((1u << lane) - 1u));
+            st.pq[c] = make_float4(my_mu, my_sg, my_P, my_th);
+            st.kr[c] = my_kr;
+            st.d0[c] = my_d0;
+            st.prev0[c] = my_pv;
+            st.comp[c] = uint8_t(lane);
+            st.wins[c] = 0;
+            st.rank0[c] = uint8_t(rank);
+            st.byrank0[BBE_INDEX(rank, 32, l.status)] = uint8_t(c);
         }
         for (int i = lane; i < NS; i += 32) {
             st.key[i] = kNoKey;
-            st.flag[i] = 0;
+            st.order[2 * i] = st.order[2 * i + 1] = uint8_t(NS);
+            st.flag[2 * i] = st.flag[2 * i + 1] = 0;
+        }
+        if (lane < 4) {
+            st.order[2 * NS + lane] = uint8_t(NS);
+            st.flag[2 * NS + lane] = 0;
         }
         const int K = MODE == 1 ? min(l.places, n) : 1;  // places run per rollout
         if constexpr (MODE == 1) {
             for (int i = lane; i < NS; i += 32) {
                 pl_n[i] = 0;
-                st.fkey[i] = kNoKey;
+                st.fsub[i] = kNoSub;
             }
             for (int i = lane; i < n * K; i += 32) pl_cnt[i] = 0;
         }
-        if (lane == 0) st.next_k = unsigned(w.k_begin) + unsigned(nseg);
+        if (lane == 0) st.next_k = k_begin + unsigned(nseg);
         __syncwarp();
 
-        const float L = b.L[r];
-        const float invL = __fdiv_rn(1.0f, L);
-        const float t0r = LAW == BBE_LAW_TIME ? b.t0[r] : 0.0f;     // time law: elapsed steps
-        const float invTr = LAW == BBE_LAW_TIME ? b.invT[r] : 0.0f;  // time law: 1 / expected duration
         const uint32_t rid = b.race_ids ? uint32_t(b.race_ids[r]) : b.race_id0 + uint32_t(r);
         // unsigned: rollout indices stay below 2^31 + 2^7
-        const unsigned kend = unsigned(w.k_begin) + unsigned(w.k_count);
+        const unsigned kend = k_begin + k_count;
 
         // per slot: segment base, competitor parameters, state, front address, rollout, block
-        int sb[V], fo[V];
-        unsigned kk[V], blk[V];
+        int fo[V];
+        unsigned blk[V];
         float mu[V], sg[V], P[V], th[V], kr[V], d[V], pv[V];
         const float4 *pqa[V];  // register-lean variant: this slot's (mu, sigma, P, theta)
         const float *kra[V];   // register-lean variant: this slot's kappa (2 rho - 1)
-        bool alive[V], pend[V], cut[V];  // running; rollout ended, to restart; stopped at max_steps
+        // a slot that runs no rollout has no position (NaN): it is never out of order, never over
+        // the line, and stays so without a test in the step
+        bool pend[V], cut[V];  // rollout ended, to restart; stopped at max_steps
+        auto alive = [&](int v) { return d[v] == d[v]; };
+        auto base = [&](int v) { return int(st.base[32 * v + lane]); };
+        // slot's stream for rollout k (competitor c of the advanced ones)
+        auto set_stream = [&](int slot, unsigned k, int c) {
+            const StreamWords q = stream_words(k, uint32_t(st.comp[c]), rid, l.round_key);
+            st.ph[slot] = make_uint4(q.d, q.e, q.f, q.g);
+            st.pha[slot] = q.a;
+        };
+        const float kDead = __int_as_float(0x7fffffff);
+        auto stop = [&](int v) {  // this slot's rollout is over
+            d[v] = kDead;
+            fo[v] = kSent;
+        };
         unsigned long long steps = 0;
         bool blk_fin = false;  // warp-uniform: some slot crossed the line in this block (a finish)
 #pragma unroll
@@ -213,10 +391,15 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             const int slot = 32 * v + lane;
             const int seg = slot / n;
             const bool used = seg < nseg;
-            sb[v] = used ? seg * n : slot;
+            const int sb = used ? seg * n : slot;
             const int c = used ? slot - seg * n : 0;
-            kk[v] = unsigned(w.k_begin) + unsigned(seg);
-            alive[v] = used && kk[v] < kend;
+            const unsigned k = k_begin + unsigned(seg);
+            const bool run = used && k < kend;
+            st.base[slot] = uint8_t(sb);
+            const int rb = 1 + (used ? seg * (n + 1) : 0);  // order[0] and flag[0] are nobody's
+            st.rbase[slot] = uint8_t(rb);
+            st.at[slot] = uint8_t(rb);
+            set_stream(slot, k, c);
             pend[v] = false;
             cut[v] = false;
             blk[v] = 0;
@@ -231,76 +414,48 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 th[v] = q.w;
                 kr[v] = st.kr[c];
             }
-            d[v] = st.d0[c];
+            d[v] = run ? st.d0[c] : kDead;
             pv[v] = st.prev0[c];
             const int r0 = st.rank0[c];
-            fo[v] = (used && r0 + 1 < n) ? BBE_INDEX(sb[v] + st.byrank0[r0 + 1], NS, l.status) * int(sizeof(float2)) : kSent;
-            if (alive[v]) {
-                st.order[BBE_INDEX(sb[v] + r0, NS, l.status)] = slot;
-                st.rnk[slot] = r0;
+            fo[v] = (run && r0 + 1 < n) ? BBE_INDEX(sb + st.byrank0[r0 + 1], NS, l.status) * int(sizeof(float2)) : kSent;
+            if (run) {
+                st.order[BBE_INDEX(rb + r0, 2 * NS + 4, l.status)] = uint8_t(slot);
+                st.at[slot] = uint8_t(rb + r0);
             }
         }
         __syncwarp();
 
-        // A segment whose rank order broke (an overtake, or equal positions): odd-even
-        // transposition by (position, slot) over the segment's rank table, then each slot's
-        // successor, and i+ for a slot level with its successor.  pb is the step's row.
+        // A segment whose rank order broke in more than isolated pairs, or with equal positions: every
+        // slot counts its rank by (position, slot), then takes its successor, or if that stands level
+        // with it the first later rank strictly in front.  pb is the step's row.
         auto full_sort = [&](const char *pb, float (&fd)[V], float (&fp)[V]) {
             const float2 *row = reinterpret_cast<const float2 *>(pb);
-            int rk[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) rk[v] = alive[v] ? st.rnk[32 * v + lane] : 0;
-            // a sort of n keys ends within n phases; 32 passes bound the loop for any input
-            for (int pass = 0; pass < 32; ++pass) {
-                bool swapped = false;
-#pragma unroll
-                for (int ph = 0; ph < 2; ++ph) {
-                    int nr[V];
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        nr[v] = rk[v];
-                        const int slot = 32 * v + lane;
-                        const bool lower = ((rk[v] ^ ph) & 1) == 0;
-                        const int pr = lower ? rk[v] + 1 : rk[v] - 1;
-                        if (alive[v] && pr >= 0 && pr < n) {
-                            const int ps = BBE_INDEX(st.order[BBE_INDEX(sb[v] + pr, NS, l.status)], NS, l.status);
-                            const float pd = row[ps].x;
-                            const bool inv = lower ? (d[v] > pd || (d[v] == pd && slot > ps))
-                                                   : (pd > d[v] || (pd == d[v] && ps > slot));
-                            if (inv) {
-                                nr[v] = pr;
-                                swapped = true;
-                            }
-                        }
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        rk[v] = nr[v];
-                        if (alive[v]) st.order[BBE_INDEX(sb[v] + nr[v], NS, l.status)] = 32 * v + lane;
-                    }
-                    __syncwarp();
-                }
-                if (!__any_sync(kAll, swapped)) break;
-            }
+            __syncwarp();
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                if (!alive[v]) continue;
-                st.rnk[32 * v + lane] = rk[v];
-                fo[v] = rk[v] + 1 < n ? BBE_INDEX(st.order[BBE_INDEX(sb[v] + rk[v] + 1, NS, l.status)], NS, l.status) *
-                                            int(sizeof(float2))
-                                      : kSent;
-                float2 f = *reinterpret_cast<const float2 *>(pb + fo[v]);
-                if (!(f.x > d[v])) {
-                    // level with the successor: the first later rank strictly in front, if any
-                    f = make_float2(INFINITY, INFINITY);
-                    for (int q = rk[v] + 2; q < n; ++q) {
-                        const float2 g = row[BBE_INDEX(st.order[BBE_INDEX(sb[v] + q, NS, l.status)], NS, l.status)];
-                        if (g.x > d[v]) {
-                            f = g;
-                            break;
-                        }
-                    }
+                const int slot = 32 * v + lane, sb = base(v);
+                int rk = 0;
+                const int end = alive(v) ? sb + n : sb;
+                for (int j = sb; j < end; ++j) {
+                    const float dj = row[BBE_INDEX(j, NS, l.status)].x;
+                    rk += dj < d[v] || (dj == d[v] && j < slot) ? 1 : 0;
+                }
+                if (alive(v)) {
+                    const int a = BBE_INDEX(int(st.rbase[slot]) + rk, 2 * NS + 3, l.status);
+                    st.order[a] = uint8_t(slot);
+                    st.at[slot] = uint8_t(a);
+                }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                if (!alive(v)) continue;
+                float2 f;
+                for (int a = int(st.at[32 * v + lane]) + 1, q = 0; q < n; ++a, ++q) {
+                    const int o = st.order[BBE_INDEX(a, 2 * NS + 4, l.status)] * int(sizeof(float2));
+                    if (q == 0) fo[v] = o;
+                    f = *reinterpret_cast<const float2 *>(pb + o);
+                    if (f.x > d[v]) break;  // the sentinel behind the last rank is
                 }
                 fd[v] = f.x;
                 fp[v] = f.y;
@@ -309,49 +464,47 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         };
 
         // The common case first: isolated overtakes.  A slot whose successor is now strictly
-        // behind it swaps ranks with that successor, unless a neighbouring pair swaps too (a
-        // chain); then every slot re-reads its successor, and what is still out of order or
+        // behind it swaps entries with that successor, unless a neighbouring pair swaps too (a
+        // chain); the slots whose successor that changed read it, and what is still out of order or
         // level goes to the full sort.
         auto repair = [&](const char *pb, float (&fd)[V], float (&fp)[V]) {
-            int rk[V];
+            int a[V];
             bool init[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                rk[v] = alive[v] ? st.rnk[32 * v + lane] : 0;
-                init[v] = alive[v] && fd[v] < d[v];
-                if (init[v]) st.flag[BBE_INDEX(sb[v] + rk[v], NS, l.status)] = 1;
+                init[v] = fd[v] < d[v];
+                a[v] = st.at[32 * v + lane];
+                if (init[v]) st.flag[a[v]] = 1;
             }
             __syncwarp();
             bool ok[V];
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-                ok[v] = init[v] && !(rk[v] > 0 && st.flag[sb[v] + rk[v] - 1]) && !(rk[v] + 2 < n && st.flag[sb[v] + rk[v] + 1]);
+            for (int v = 0; v < V; ++v) ok[v] = init[v] && st.flag[a[v] - 1] == 0 && st.flag[a[v] + 1] == 0;
             __syncwarp();
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 if (!init[v]) continue;
-                st.flag[sb[v] + rk[v]] = 0;
+                st.flag[a[v]] = 0;
                 if (ok[v]) {
-                    const int slot = 32 * v + lane;
-                    const int f = BBE_INDEX(st.order[BBE_INDEX(sb[v] + rk[v] + 1, NS, l.status)], NS, l.status);
-                    st.order[sb[v] + rk[v]] = f;
-                    st.order[sb[v] + rk[v] + 1] = slot;
-                    st.rnk[f] = rk[v];
-                    st.rnk[slot] = rk[v] + 1;
+                    const int f = BBE_INDEX(fo[v] / int(sizeof(float2)), NS, l.status);
+                    st.order[a[v]] = uint8_t(f);
+                    st.order[a[v] + 1] = uint8_t(32 * v + lane);
+                    st.at[f] = uint8_t(a[v]);
+                    st.at[32 * v + lane] = uint8_t(a[v] + 1);
                 }
             }
             __syncwarp();
             bool again = false;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                if (!alive[v]) continue;
-                const int r1 = st.rnk[32 * v + lane] + 1;
-                fo[v] = r1 < n ? BBE_INDEX(st.order[BBE_INDEX(sb[v] + r1, NS, l.status)], NS, l.status) * int(sizeof(float2))
-                               : kSent;
-                const float2 f = *reinterpret_cast<const float2 *>(pb + fo[v]);
-                fd[v] = f.x;
-                fp[v] = f.y;
-                again |= !(f.x > d[v]);
+                const int o = st.order[BBE_INDEX(int(st.at[32 * v + lane]) + 1, 2 * NS + 4, l.status)] * int(sizeof(float2));
+                if (o != fo[v] && alive(v)) {
+                    fo[v] = o;
+                    const float2 f = *reinterpret_cast<const float2 *>(pb + o);
+                    fd[v] = f.x;
+                    fp[v] = f.y;
+                }
+                again |= fd[v] <= d[v];
             }
             if (__any_sync(kAll, again)) full_sort(pb, fd, fp);
         };
@@ -368,16 +521,20 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             __syncwarp();
             {
                 unsigned long long fk[V];
+                int sb[V];
                 bool more = false;
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
                     const int slot = 32 * v + lane;
-                    fk[v] = st.fkey[slot];
-                    if (fk[v] != kNoKey) {
+                    sb[v] = base(v);
+                    const unsigned sub = st.fsub[slot];
+                    fk[v] = kNoKey;
+                    if (sub != kNoSub) {
                         const float2 c = st.fcross[slot];
                         const float tau = __fdiv_rn(__fsub_rn(L, c.x), c.y);
-                        fk[v] |= static_cast<unsigned long long>(__float_as_uint(tau)) << 8;
-                        st.fkey[slot] = kNoKey;
+                        fk[v] = (static_cast<unsigned long long>(sub) << 40) |
+                                (static_cast<unsigned long long>(__float_as_uint(tau)) << 8) | unsigned(slot);
+                        st.fsub[slot] = kNoSub;
                         more = true;
                     }
                 }
@@ -392,10 +549,10 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     for (int v = 0; v < V; ++v) {
                         won[v] = fk[v] != kNoKey && st.key[sb[v]] == fk[v];
                         if (won[v]) {
-                            const int p = BBE_INDEX(pl_n[sb[v]], n, l.status);
-                            pl_ord[sb[v] + p] = 32 * v + lane - sb[v];
-                            pl_n[sb[v]] = p + 1;
-                            if (p == K - 1) pl_kj[sb[v]] = int(fk[v] >> 40);
+                            const int p = BBE_INDEX(int(pl_n[sb[v]]), n, l.status);
+                            pl_ord[sb[v] + p] = uint8_t(32 * v + lane - sb[v]);
+                            pl_n[sb[v]] = uint8_t(p + 1);
+                            if (p == K - 1) pl_kj[sb[v]] = uint8_t(fk[v] >> 40);
                         }
                     }
                     __syncwarp();
@@ -411,18 +568,18 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                if (!alive[v] && !cut[v]) continue;
-                const int slot = 32 * v + lane;
-                const int jend = pl_n[sb[v]] >= K ? pl_kj[sb[v]] : -1;  // sub-step of the K-th place
+                if (!alive(v) && !cut[v]) continue;
+                const int slot = 32 * v + lane, sb = base(v);
+                const int jend = pl_n[sb] >= K ? pl_kj[sb] : -1;  // sub-step of the K-th place
                 if (jend >= 0) {
-                    if (slot == sb[v]) steps += (unsigned long long)(blk[v] * 4u + unsigned(jend) + 1u);
+                    if (slot == sb) steps += (unsigned long long)(blk[v] * 4u + unsigned(jend) + 1u);
                     pend[v] = true;
                 } else if (cut[v]) {
-                    if (slot == sb[v]) steps += (unsigned long long)l.max_steps;
-                    hit_limit = true;
+                    if (slot == sb) steps += (unsigned long long)l.max_steps;
+                    atomicOr(l.status, kStatusStepLimit);
                     pend[v] = true;
                 }
-                alive[v] = alive[v] && !pend[v];
+                if (pend[v]) stop(v);
                 cut[v] = false;
             }
             __syncwarp();
@@ -436,14 +593,15 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         auto tally_completed = [&]() {
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                if (!pend[v] || pl_n[sb[v]] < K) continue;
-                const int c = 32 * v + lane - sb[v];  // this slot's competitor
-                if (c < K) atomicAdd(&pl_cnt[BBE_INDEX(pl_ord[sb[v] + c] * K + c, n * K, l.status)], 1);
+                const int sb = base(v);
+                if (!pend[v] || pl_n[sb] < K) continue;
+                const int c = 32 * v + lane - sb;  // this slot's competitor
+                if (c < K) atomicAdd(&pl_cnt[BBE_INDEX(pl_ord[sb + c] * K + c, n * K, l.status)], 1);
                 if (c == 0 && (l.orders != nullptr || l.hist_keys != nullptr)) {
                     unsigned code = 0u, taken = 0u;
                     unsigned long long key = 0ull;
                     for (int j = 0; j < K; ++j) {
-                        const int cj = pl_ord[sb[v] + j];
+                        const int cj = pl_ord[sb + j];
                         code = code * unsigned(n) + unsigned(cj);
                         key = key * unsigned(n - j) + unsigned(__popc(((1u << cj) - 1u) & ~taken));
                         taken |= 1u << cj;
@@ -464,23 +622,25 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             __syncwarp();
         };
 
-        // One step of every slot: sub-step J of the Philox block (its normal is z[v][J]); CHK
-        // when some segment may reach max_steps within the block.
+        // One step of every slot: sub-step j0 + J of the Philox block (its normal is z[v][J]); CHK
+        // when some segment may reach its limit within the block.
+        int j0 = 0;
         auto step = [&](auto Jc, auto CHKc, const float (&z)[V][4]) {
-            constexpr int J = decltype(Jc)::value;
+            const int J = Jc;  // a compile-time constant, but for the rare checked block
             constexpr bool CHK = decltype(CHKc)::value;
-            constexpr int BO = (J & 1) * ROWB;
+            const int BO = (J & 1) * ROWB;
             if constexpr (CHK) {
                 // a rollout reaching step max_steps stops there and counts for nobody (in place
                 // mode unless it ended earlier in the block, decided at the block's end)
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
-                    if (alive[v] && int(blk[v]) * 4 + J >= l.max_steps) {
-                        alive[v] = false;
+                    if (alive(v) && int(blk[v]) * 4 + J >= limit) {
+                        stop(v);
                         if constexpr (MODE == 0) {
                             pend[v] = true;
-                            hit_limit = true;
-                            if (32 * v + lane == sb[v]) steps += (unsigned long long)l.max_steps;
+                            if (limit < l.max_steps) redo = true;
+                            else atomicOr(l.status, kStatusStepLimit);
+                            if (32 * v + lane == base(v)) steps += (unsigned long long)l.max_steps;
                         } else {
                             cut[v] = true;
                         }
@@ -499,7 +659,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 const float2 f = *reinterpret_cast<const float2 *>(posb + BO + BBE_INDEX(fo[v], kSent + 1, l.status));
                 fd[v] = f.x;
                 fp[v] = f.y;
-                bad |= alive[v] && !(f.x > d[v]);
+                bad |= f.x <= d[v];
             }
             if (__any_sync(kAll, bad)) repair(posb + BO, fd, fp);
             // Eq. 1 (a successor at +inf is never within theta: the free branch)
@@ -522,14 +682,14 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     thv = th[v];
                     kv = kr[v];
                 }
-                const float Rc = responsiveness<LAW>(kv, d[v], invL, t0r, int(blk[v]) * 4 + J, invTr);
+                const float Rc = responsiveness<LAW>(kv, d[v], invL, t0r, int(blk[v]) * 4 + j0 + J, invTr);
                 const bool blocked = !(__fsub_rn(fd[v], d[v]) > thv);
                 float Sv = blocked ? __fmul_rn(Rc, fminf(pv[v], fp[v]))
-                                   : __fmul_rn(__fmul_rn(Rc, Pv), __fmaf_rn(sgv, z[v][J], muv));
+                                   : __fmul_rn(__fmul_rn(Rc, Pv), __fmaf_rn(sgv, J == 0 ? z[v][0] : J == 1 ? z[v][1] : J == 2 ? z[v][2] : z[v][3], muv));
                 Sv = fmaxf(Sv, kStepFloor);
                 S[v] = Sv;
                 dn[v] = __fadd_rn(d[v], Sv);
-                fv[v] = alive[v] && dn[v] >= L && (MODE == 0 || d[v] < L);
+                fv[v] = dn[v] >= L && (MODE == 0 || d[v] < L);
                 fin |= fv[v];
             }
             if constexpr (MODE == 1) {
@@ -543,7 +703,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     for (int v = 0; v < V; ++v) {
                         if (fv[v]) {
                             // tau joins the key at the block's end (one division there, none here)
-                            st.fkey[32 * v + lane] = (static_cast<unsigned long long>(J) << 40) | unsigned(32 * v + lane);
+                            st.fsub[32 * v + lane] = uint8_t(j0 + J);
                             st.fcross[32 * v + lane] = make_float2(d[v], S[v]);
                         }
                     }
@@ -556,28 +716,30 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 for (int v = 0; v < V; ++v) {
                     if (fv[v]) {
                         const float tau = __fdiv_rn(__fsub_rn(L, d[v]), S[v]);
-                        atomicMin(&st.key[sb[v]], (static_cast<unsigned long long>(__float_as_uint(tau)) << 32) |
+                        atomicMin(&st.key[base(v)], (static_cast<unsigned long long>(__float_as_uint(tau)) << 32) |
                                                       unsigned(32 * v + lane));
                     }
                 }
                 __syncwarp();
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
-                    if (alive[v]) {
-                        const unsigned long long kw = st.key[sb[v]];
+                    if (alive(v)) {
+                        const int sb = base(v);
+                        const unsigned long long kw = st.key[sb];
                         if (kw != kNoKey) {
                             const int slot = 32 * v + lane;
-                            if (int(unsigned(kw)) == slot) atomicAdd(&st.wins[BBE_INDEX(slot - sb[v], 32, l.status)], 1);
-                            alive[v] = false;
+                            if (int(unsigned(kw)) == slot) atomicAdd(&st.wins[BBE_INDEX(slot - sb, 32, l.status)], 1);
+                            dn[v] = kDead;
+                            fo[v] = kSent;
                             pend[v] = true;
-                            if (slot == sb[v]) steps += (unsigned long long)(blk[v] * 4u + unsigned(J) + 1u);
+                            if (slot == sb) steps += (unsigned long long)(blk[v] * 4u + unsigned(j0 + J) + 1u);
                         }
                     }
                 }
                 __syncwarp();
 #pragma unroll
                 for (int v = 0; v < V; ++v)
-                    if (fv[v]) st.key[sb[v]] = kNoKey;
+                    if (fv[v]) st.key[base(v)] = kNoKey;
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -587,7 +749,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         };
 
         // blocks before one in which a rollout could reach max_steps (the check starts there)
-        unsigned left = l.max_steps >= 4 ? unsigned(l.max_steps - 4) / 4u + 1u : 0u;
+        unsigned left = limit >= 4 ? unsigned(limit - 4) / 4u + 1u : 0u;
         // warp-uniform: the last block may have changed which slots run (a finish, a cut-off);
         // after a block without either the reduction below would find nothing to do
         bool blk_event = true;
@@ -600,41 +762,41 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 pany |= pend[v];
-                aany |= alive[v];
+                aany |= alive(v);
             }
             const unsigned state = __reduce_or_sync(kAll, (pany ? 1u : 0u) | (aany ? 2u : 0u));
             if (state & 1u) {
                 if constexpr (MODE == 1) tally_completed();
 #pragma unroll
                 for (int v = 0; v < V; ++v)
-                    if (pend[v] && 32 * v + lane == sb[v]) {
-                        st.segk[sb[v]] = atomicAdd(&st.next_k, 1u);
-                        if constexpr (MODE == 1) pl_n[sb[v]] = 0;
+                    if (pend[v] && 32 * v + lane == base(v)) {
+                        st.segk[32 * v + lane] = atomicAdd(&st.next_k, 1u);
+                        if constexpr (MODE == 1) pl_n[32 * v + lane] = 0;
                     }
                 __syncwarp();
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
                     if (!pend[v]) continue;
                     pend[v] = false;
-                    const unsigned knew = st.segk[sb[v]];
+                    const int slot = 32 * v + lane, sb = base(v);
+                    const unsigned knew = st.segk[sb];
                     if (knew < kend) {
-                        const int slot = 32 * v + lane;
-                        const int c = slot - sb[v];
-                        kk[v] = knew;
-                        alive[v] = true;
+                        const int c = slot - sb;
+                        set_stream(slot, knew, c);
                         blk[v] = 0;
                         d[v] = st.d0[c];
                         pv[v] = st.prev0[c];
                         const int r0 = st.rank0[c];
-                        fo[v] = r0 + 1 < n ? (sb[v] + st.byrank0[r0 + 1]) * int(sizeof(float2)) : kSent;
-                        st.order[sb[v] + r0] = slot;
-                        st.rnk[slot] = r0;
+                        fo[v] = r0 + 1 < n ? (sb + st.byrank0[r0 + 1]) * int(sizeof(float2)) : kSent;
+                        const int a = st.rbase[slot] + r0;
+                        st.order[a] = uint8_t(slot);
+                        st.at[slot] = uint8_t(a);
                     }
                 }
                 __syncwarp();
                 bool any_alive = false;
 #pragma unroll
-                for (int v = 0; v < V; ++v) any_alive |= alive[v];
+                for (int v = 0; v < V; ++v) any_alive |= alive(v);
                 if (!__any_sync(kAll, any_alive)) break;
             } else if (!(state & 2u)) {
                 break;
@@ -645,29 +807,49 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             float z[V][4];
 #pragma unroll
             for (int v = 0; v < V; ++v)
-                draw_block<DIST>(kk[v], blk[v], uint32_t(32 * v + lane - sb[v]), rid, l.round_key, z[v]);
+                draw_block<DIST>(st.ph[32 * v + lane], st.pha[32 * v + lane], blk[v], l.round_key, z[v]);
             // no slot is further into its rollout than the blocks the work item has run, so a
             // warp-uniform count-down rules out the step limit in all but the longest items
             bool near_limit = false;
             if (left == 0u) {
 #pragma unroll
-                for (int v = 0; v < V; ++v) near_limit |= alive[v] && int(blk[v]) * 4 + 4 > l.max_steps;
+                for (int v = 0; v < V; ++v) near_limit |= alive(v) && int(blk[v]) * 4 + 4 > limit;
             } else {
                 --left;
             }
             blk_fin = false;
             if (left == 0u && __any_sync(kAll, near_limit)) {
                 blk_event = true;
-                step(std::integral_constant<int, 0>{}, std::true_type{}, z);
-                step(std::integral_constant<int, 1>{}, std::true_type{}, z);
-                step(std::integral_constant<int, 2>{}, std::true_type{}, z);
-                step(std::integral_constant<int, 3>{}, std::true_type{}, z);
+#pragma unroll 1
+                for (int J = 0; J < 4; ++J) step(J, std::true_type{}, z);
                 if constexpr (MODE == 1) block_end();
+                else if (__any_sync(kAll, redo)) break;
             } else {
-                step(std::integral_constant<int, 0>{}, std::false_type{}, z);
-                step(std::integral_constant<int, 1>{}, std::false_type{}, z);
-                step(std::integral_constant<int, 2>{}, std::false_type{}, z);
-                step(std::integral_constant<int, 3>{}, std::false_type{}, z);
+                if constexpr (MODE == 0) {
+                    // two copies of the step, run twice (the second time with the block's other two
+                    // normals): with four, the step, its repair and its finish overflow the
+                    // instruction cache where overtakes are frequent (700 bunched races of 13: 19.4
+                    // instead of 15.8 ms; spread races without overtakes lose 2 %)
+                    j0 = 0;
+#pragma unroll 1
+                    for (;;) {
+                        step(std::integral_constant<int, 0>{}, std::false_type{}, z);
+                        step(std::integral_constant<int, 1>{}, std::false_type{}, z);
+                        if (j0 != 0) break;
+                        j0 = 2;
+#pragma unroll
+                        for (int v = 0; v < V; ++v) {
+                            z[v][0] = z[v][2];
+                            z[v][1] = z[v][3];
+                        }
+                    }
+                    j0 = 0;
+                } else {
+                    step(std::integral_constant<int, 0>{}, std::false_type{}, z);
+                    step(std::integral_constant<int, 1>{}, std::false_type{}, z);
+                    step(std::integral_constant<int, 2>{}, std::false_type{}, z);
+                    step(std::integral_constant<int, 3>{}, std::false_type{}, z);
+                }
                 if constexpr (MODE == 1) {
                     if (blk_fin) block_end();
                 }
@@ -677,6 +859,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             for (int v = 0; v < V; ++v) ++blk[v];
         }
 
+        if (MODE == 0 && __any_sync(kAll, redo)) continue;
         // one global atomic per competitor with wins (per competitor and place in place mode), one
         // per work item for the step total
         __syncwarp();
@@ -686,21 +869,22 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 if (cc != 0) atomicAdd(&l.counts[(off + i / K) * l.places + i % K], cc);
             }
         } else {
-            if (lane < n && st.wins[lane] != 0) atomicAdd(&l.counts[off + lane], st.wins[lane]);
+            if (lane < n && st.wins[lane] != 0) atomicAdd(&l.counts[off + st.comp[lane]], st.wins[lane]);
         }
         for (int o = 16; o > 0; o >>= 1) steps += __shfl_xor_sync(kAll, steps, o);
         if (lane == 0 && l.steps != nullptr) atomicAdd(l.steps + r, steps);
+        break;
+        }
     }
-    if (__any_sync(kAll, hit_limit) && lane == 0) atomicOr(l.status, kStatusStepLimit);
 }
 
 // Dynamic shared memory of a block: the warps' stages, then in place mode each warp's place
-// lists (3 x 32 V ints) and [competitor][place] table (place_cells ints).
+// lists (3 x 32 V bytes) and [competitor][place] table (place_cells ints).
 template <int V, int MODE>
 size_t win_stage_bytes(int block, int place_cells)
 {
     const size_t warps = size_t(block / 32);
-    return warps * sizeof(WinStage<V>) + (MODE == 1 ? warps * (3 * 32 * V + size_t(place_cells)) * sizeof(int) : 0);
+    return warps * sizeof(WinStage<V>) + (MODE == 1 ? warps * (3 * 8 * V + size_t(place_cells)) * sizeof(int) : 0);
 }
 
 // The largest place table a launch may ask for (32 competitors x 32 places).
