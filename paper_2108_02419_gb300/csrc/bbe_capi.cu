@@ -59,8 +59,8 @@ bool is_host_memory(const void *p)
 }
 
 // copy caller memory (host or device) into a host vector: memcpy for host memory, an
-// asynchronous device-to-host copy otherwise (the caller synchronises the stream)
-bbe_status copy_in(void *dst, const void *src, size_t bytes, cudaStream_t s, const char *what)
+// asynchronous device-to-host copy otherwise (sets *pending: the caller synchronises the stream)
+bbe_status copy_in(void *dst, const void *src, size_t bytes, cudaStream_t s, const char *what, bool *pending = nullptr)
 {
     if (bytes == 0) return BBE_OK;
     if (is_host_memory(src)) {
@@ -68,6 +68,7 @@ bbe_status copy_in(void *dst, const void *src, size_t bytes, cudaStream_t s, con
         return BBE_OK;
     }
     cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s);
+    if (pending) *pending = true;
     if (e != cudaSuccess) {
         set_error(std::string("copy of ") + what + ": " + cudaGetErrorString(e));
         return BBE_ERR_CUDA;
@@ -197,9 +198,11 @@ struct ItemRun {
 };
 
 // items[i] for every list index i: the run holding i (the last whose first index is at most i,
-// by binary search over the runs in list order), then its item i - first.
+// by binary search over the runs in list order), then its item i - first.  With records of several
+// races (full > 0) a run holds all races of its record, `full` items each up to index full_end and one
+// each (the remainders) from there on.
 __global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, int32_t total, bool tickets,
-                             bbe::WorkItem *__restrict__ items)
+                             int32_t full, int32_t full_end, bbe::WorkItem *__restrict__ items)
 {
     const int32_t i = int32_t(blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= total) return;
@@ -210,11 +213,18 @@ __global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, i
         else hi = mid - 1;
     }
     const ItemRun r = runs[lo];
-    items[i] = bbe::WorkItem{r.race, tickets ? r.k0 : r.k0 + (i - r.first) * r.chunk, r.chunk, 0};
+    int32_t race = r.race, j = i - r.first;
+    if (full > 0) {
+        const int32_t each = i < full_end ? full : 1;
+        race += j / each;
+        j %= each;
+    }
+    items[i] = bbe::WorkItem{race, tickets ? r.k0 : r.k0 + j * r.chunk, r.chunk, 0};
 }
 
 bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
 {
+    const int32_t n_rec = b->n_races / b->reps;  // host records, each of `reps` equal races
     // Per race: full chunks of `chunk` rollouts (all of one cost) and a remainder.  The list puts
     // longer work first: full chunks race by race in descending cost per chunk, then the
     // remainders in descending cost.  Sorting races rather than items keeps the host work
@@ -227,7 +237,7 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
     std::vector<RacePlan> plans[kGroups];
     // keep the whole list near kMaxItems items: very large batches get larger items
     int64_t total_rollouts = 0;
-    for (int r = 0; r < b->n_races; ++r) total_rollouts += b->h_R[r];
+    for (int r = 0; r < n_rec; ++r) total_rollouts += b->h_R[r] * b->reps;
     const int64_t min_chunk = (total_rollouts + kMaxItems - 1) / kMaxItems;
     int64_t race_items = kMaxItemsPerRace;  // items per race at most (lifted for very small batches)
     auto chunk_of = [&](int r, int64_t per_lane, int nseg) {
@@ -246,9 +256,9 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
     const int64_t warp_slots = int64_t(std::max(1, b->num_sms)) * 64;
     auto items_at = [&](int64_t pl) {  // items of the list at pl rollouts per lane, counted up to warp_slots
         int64_t items = 0;
-        for (int r = 0; r < b->n_races && items < warp_slots; ++r) {
+        for (int r = 0; r < n_rec && items < warp_slots; ++r) {
             const int64_t chunk = chunk_of(r, pl, nseg_of(r));
-            items += (b->h_R[r] + chunk - 1) / chunk;
+            items += (b->h_R[r] + chunk - 1) / chunk * b->reps;
         }
         return items;
     };
@@ -278,7 +288,7 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
     // others waiting at the end
     b->most = int32_t(std::min<int64_t>(INT32_MAX, std::max<int64_t>(1, total_rollouts / (int64_t(std::max(1, b->num_sms)) * 28 * 4))));
     size_t total = 0;
-    for (int r = 0; r < b->n_races; ++r) {
+    for (int r = 0; r < n_rec; ++r) {
         const int n = b->h_off[r + 1] - b->h_off[r];
         const int v = slots_for(n, b->cfg.slots_per_lane, b->slots_by_n, b->default_slots);
         const int nseg = nseg_of(r);
@@ -287,7 +297,7 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
         RacePlan pl{r, chunk, b->h_R[r] / chunk, b->h_R[r] % chunk, b->h_k0.empty() ? 0 : b->h_k0[r], 0.0, 0.0};
         pl.cost_full = double((chunk + nseg - 1) / nseg) * st;
         pl.cost_rem = double((pl.rem + nseg - 1) / nseg) * st;
-        total += size_t(pl.full) + (pl.rem > 0 ? 1 : 0);
+        total += (size_t(pl.full) + (pl.rem > 0 ? 1 : 0)) * size_t(b->reps);
         plans[group_of(v)].push_back(pl);
     }
     if (total > size_t(INT32_MAX)) {
@@ -297,26 +307,32 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
     // the list as runs of equal items (a race's full chunks, then its remainder), expanded into
     // items on the device: 16 bytes per run cross the bus instead of 16 per item
     std::vector<ItemRun> runs;
-    runs.reserve(size_t(2) * size_t(b->n_races));
-    int32_t listed = 0;
+    runs.reserve(size_t(2) * size_t(n_rec));
+    int32_t listed = 0, full_end = 0;  // full_end: with several races a record, all in one group
     for (int g = 0; g < kGroups; ++g) {
         std::vector<RacePlan> &pg = plans[g];
         const int32_t before = listed;
         std::stable_sort(pg.begin(), pg.end(), [](const RacePlan &x, const RacePlan &y) { return x.cost_full > y.cost_full; });
         for (const RacePlan &pl : pg) {
             if (pl.full == 0) continue;
-            runs.push_back(ItemRun{pl.race, int32_t(pl.k0), int32_t(pl.chunk), listed});
-            listed += int32_t(pl.full);
+            runs.push_back(ItemRun{pl.race * b->reps, int32_t(pl.k0), int32_t(pl.chunk), listed});
+            listed += int32_t(pl.full) * b->reps;
         }
+        if (b->reps > 1 && !pg.empty()) full_end = listed;
         std::stable_sort(pg.begin(), pg.end(), [](const RacePlan &x, const RacePlan &y) { return x.cost_rem > y.cost_rem; });
         for (const RacePlan &pl : pg) {
             if (pl.rem == 0) continue;
-            if (b->tickets) runs.push_back(ItemRun{pl.race, int32_t(pl.k0), int32_t(pl.chunk), listed});
-            else runs.push_back(ItemRun{pl.race, int32_t(pl.k0 + pl.full * pl.chunk), int32_t(pl.rem), listed});
-            listed += 1;
+            if (b->tickets) runs.push_back(ItemRun{pl.race * b->reps, int32_t(pl.k0), int32_t(pl.chunk), listed});
+            else runs.push_back(ItemRun{pl.race * b->reps, int32_t(pl.k0 + pl.full * pl.chunk), int32_t(pl.rem), listed});
+            listed += b->reps;
         }
         b->n_items_v[g] = listed - before;
     }
+
+    int32_t full = 0;  // items of full chunks per race, the same for all races of a batch with such records
+    if (b->reps > 1)
+        for (int g = 0; g < kGroups; ++g)
+            if (!plans[g].empty()) full = int32_t(std::max<int64_t>(1, plans[g][0].full));
 
     // the new list is in place before the call returns (made on `upload`, the staging call's
     // stream, else on the batch's free stream); the old one is freed behind this batch's work
@@ -331,7 +347,8 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
     if (!runs.empty()) {
         BBE_CUDA_TRY(pool_alloc(reinterpret_cast<void **>(&d_runs), runs.size() * sizeof(ItemRun), upload));
         BBE_CUDA_TRY(cudaMemcpyAsync(d_runs, runs.data(), runs.size() * sizeof(ItemRun), cudaMemcpyHostToDevice, upload));
-        expand_items<<<unsigned((listed + 255) / 256), 256, 0, upload>>>(d_runs, int32_t(runs.size()), listed, b->tickets, fresh);
+        expand_items<<<unsigned((listed + 255) / 256), 256, 0, upload>>>(d_runs, int32_t(runs.size()), listed, b->tickets, full,
+                                                                            full_end, fresh);
         BBE_CUDA_TRY(cudaGetLastError());
         BBE_CUDA_TRY(cudaFreeAsync(d_runs, upload));
     }
@@ -457,6 +474,55 @@ bbe_status ensure_graph(bbe_batch *b, int32_t *counts, int64_t *steps)
     return BBE_OK;
 }
 
+// The state of every record (Section 3: S > 0, P in [0,1], positions on the track); sets the error.
+bbe_status check_state(const bbe_batch *b)
+{
+    for (int r = 0; r < b->n_races / b->reps; ++r) {
+        const float L = b->h_L[r];
+        if (!finite(L) || !(L > 0.0f)) {
+            set_error("track_len of race " + std::to_string(r * b->reps) + " is not a positive finite number");
+            return BBE_ERR_ARG;
+        }
+        if (b->h_R[r] < 1 || b->h_R[r] > INT32_MAX) {
+            set_error("rollouts of race " + std::to_string(r * b->reps) + " outside 1..2^31-1");
+            return BBE_ERR_ARG;
+        }
+        for (int i = b->h_off[r]; i < b->h_off[r + 1]; ++i) {
+            const float d = b->h_d0[i];
+            auto where = [&]() { return " (race " + std::to_string(r * b->reps) + ", competitor " + std::to_string(i - b->h_off[r]) + ")"; };
+            if (!finite(d) || d < 0.0f) {
+                set_error("position must be finite and >= 0" + where());
+                return BBE_ERR_ARG;
+            }
+            if (d >= L) {
+                set_error("competitor already finished (d >= L)" + where());
+                return BBE_ERR_FINISHED;
+            }
+            if (!finite(b->h_mu[i]) || !(b->h_mu[i] > 0.0f) || !finite(b->h_sigma[i]) || !(b->h_sigma[i] >= 0.0f)) {
+                set_error("need finite mu > 0 and sigma >= 0" + where());
+                return BBE_ERR_ARG;
+            }
+            if (!(b->h_rho[i] >= 0.0f && b->h_rho[i] <= 1.0f)) {
+                set_error("responsiveness rho outside [0, 1]" + where());
+                return BBE_ERR_ARG;
+            }
+            if (!(b->h_P[i] > 0.0f && b->h_P[i] <= 1.0f)) {
+                set_error("preference P outside (0, 1]" + where());
+                return BBE_ERR_ARG;
+            }
+            if (!finite(b->h_theta[i]) || !(b->h_theta[i] >= 0.0f)) {
+                set_error("theta must be finite and >= 0" + where());
+                return BBE_ERR_ARG;
+            }
+            if (!b->h_prev.empty() && (!finite(b->h_prev[i]) || !(b->h_prev[i] > 0.0f))) {
+                set_error("prev_step must be finite and > 0" + where());
+                return BBE_ERR_ARG;
+            }
+        }
+    }
+    return BBE_OK;
+}
+
 template <typename T>
 T *carve(char *&p, size_t count)
 {
@@ -465,7 +531,188 @@ T *carve(char *&p, size_t count)
     return out;
 }
 
+// One device arena for a staged batch.
+struct Arena {
+    size_t bytes;
+    int32_t *off;
+    float *L;
+    int64_t *R;
+    int32_t *cr, *ids;
+    float *d0, *mu, *sigma, *rho, *P, *theta, *prev;
+};
+
+bbe_status make_arena(bbe_batch *b, Arena &A, cudaStream_t s)
+{
+    const size_t n_races = size_t(b->n_races), nt = size_t(b->n_total);
+    size_t bytes = 0;
+    auto add = [&](size_t n) { bytes += (n + 255) / 256 * 256; };
+    add((n_races + 1) * 4); add(n_races * 4); add(n_races * 8); add(nt * 4); add(n_races * 4);
+    for (int i = 0; i < 7; ++i) add(nt * 4);
+    add((kGroups + 1 + n_races) * 4);
+    cudaError_t e = cudaGetDevice(&b->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device);
+    if (e == cudaSuccess) e = pool_alloc(&b->arena, bytes, s);
+    if (e != cudaSuccess) {
+        set_error(std::string("device allocation: ") + cudaGetErrorString(e));
+        return BBE_ERR_CUDA;
+    }
+    char *p = static_cast<char *>(b->arena);
+    A.bytes = bytes;
+    A.off = carve<int32_t>(p, n_races + 1);
+    A.L = carve<float>(p, n_races);
+    A.R = carve<int64_t>(p, n_races);
+    A.cr = carve<int32_t>(p, nt);
+    A.ids = carve<int32_t>(p, n_races);
+    for (float **q : {&A.d0, &A.mu, &A.sigma, &A.rho, &A.P, &A.theta, &A.prev}) *q = carve<float>(p, nt);
+    b->d_queue = carve<int32_t>(p, kGroups + 1 + n_races);
+    b->d_status = b->d_queue + kGroups;
+    b->d_next = b->d_status + 1;
+    return BBE_OK;
+}
+
+void default_launch(bbe_batch *b)
+{
+    b->cfg = bbe_launch_cfg{kDefaultWarpsPerBlock, kDefaultBlocksPerSm, kDefaultRolloutsPerLane, BBE_MAX_STEPS_DEFAULT, 0};
+    for (int g = 0; g < kGroups; ++g)
+        b->resident[g] = bbe::rollout_resident_blocks(b->dist, kSlots[g], 32 * kDefaultWarpsPerBlock);
+}
+
+std::atomic<uint64_t> g_next_serial{1};
+
+// The arrays of a repeated batch from its records (rec: d0, mu, sigma, rho, P, theta, prev of n_rec x n
+// competitors, then t0 of the n_rec records if t0 is to be written): one thread per competitor.
+struct Repeat {
+    int32_t n_races, nt, reps, n, n_rec;
+    float L, invT;
+    int64_t R;
+    const float *rec;
+    float *t0, *invTs;  // or null
+    Arena a;
+};
+
+__global__ void repeat_records(Repeat q)
+{
+    const int32_t i = int32_t(blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= q.nt) return;
+    const int32_t r = i / q.n, c = i - r * q.n, k = r / q.reps, m = q.n_rec * q.n;
+    const float *src = q.rec + k * q.n + c;
+    q.a.cr[i] = r;
+    q.a.d0[i] = src[0];
+    q.a.mu[i] = src[m];
+    q.a.sigma[i] = src[2 * m];
+    q.a.rho[i] = src[3 * m];
+    q.a.P[i] = src[4 * m];
+    q.a.theta[i] = src[5 * m];
+    q.a.prev[i] = src[6 * m];
+    if (c != 0) return;
+    q.a.off[r] = i;
+    q.a.L[r] = q.L;
+    q.a.R[r] = q.R;
+    if (r == q.n_races - 1) q.a.off[q.n_races] = q.nt;
+    if (q.t0 != nullptr) {
+        q.t0[r] = q.rec[7 * m + k];
+        q.invTs[r] = q.invT;
+    }
+}
+
 }  // namespace
+
+void bbe::unfold(const bbe_batch *cb)
+{
+    bbe_batch *b = const_cast<bbe_batch *>(cb);
+    std::lock_guard<std::mutex> g(b->unfold_mu);
+    if (b->reps == 1) return;
+    const size_t reps = size_t(b->reps), n_rec = size_t(b->n_races) / reps, n = size_t(b->max_n);  // all of n
+    auto each = [&](auto &v, size_t block) {
+        if (v.empty()) return;
+        auto w = std::remove_reference_t<decltype(v)>();
+        w.reserve(v.size() * reps);
+        for (size_t k = 0; k < n_rec; ++k)
+            for (size_t j = 0; j < reps; ++j) w.insert(w.end(), v.begin() + k * block, v.begin() + (k + 1) * block);
+        v = std::move(w);
+    };
+    for (auto *v : {&b->h_d0, &b->h_mu, &b->h_sigma, &b->h_rho, &b->h_P, &b->h_theta, &b->h_prev}) each(*v, n);
+    for (auto *v : {&b->h_L, &b->h_t0, &b->h_T}) each(*v, 1);
+    each(b->h_R, 1);
+    b->h_off.resize(size_t(b->n_races) + 1);
+    for (size_t r = 0; r < b->h_off.size(); ++r) b->h_off[r] = int32_t(r * n);
+    b->reps = 1;
+}
+
+bbe_status bbe::stage_repeated(bbe_batch **out, int32_t n_rec, int32_t reps, int32_t n, float L, int64_t R,
+                               std::vector<float> d0, std::vector<float> mu, std::vector<float> sigma,
+                               std::vector<float> rho, std::vector<float> P, std::vector<float> theta,
+                               std::vector<float> prev, uint64_t seed, bbe_dist dist, uint32_t race_id0,
+                               const std::vector<float> *t0, float T, cudaStream_t s)
+{
+    // The records alone are checked, planned and sent; a kernel repeats them (121 snapshots of 1000
+    // bettors: 25 MB that the host would build, check and copy, 17 ms of a 25 ms pass).
+    *out = nullptr;
+    const size_t m = size_t(n_rec) * size_t(n);
+    auto b = new bbe_batch();
+    b->serial = g_next_serial.fetch_add(1);
+    b->n_races = n_rec * reps;
+    b->n_total = b->n_races * n;
+    b->max_n = n;
+    b->seed = seed;
+    b->dist = int32_t(dist);
+    b->race_id0 = race_id0;
+    b->reps = reps;
+    b->h_off.resize(size_t(n_rec) + 1);
+    for (size_t r = 0; r < b->h_off.size(); ++r) b->h_off[r] = int32_t(r) * n;
+    b->h_L.assign(size_t(n_rec), L);
+    b->h_R.assign(size_t(n_rec), R);
+    std::vector<float> rec;
+    rec.reserve(7 * m + size_t(n_rec));
+    for (auto *v : {&d0, &mu, &sigma, &rho, &P, &theta, &prev}) rec.insert(rec.end(), v->begin(), v->end());
+    if (t0) rec.insert(rec.end(), t0->begin(), t0->end());
+    b->h_d0 = std::move(d0);
+    b->h_mu = std::move(mu);
+    b->h_sigma = std::move(sigma);
+    b->h_rho = std::move(rho);
+    b->h_P = std::move(P);
+    b->h_theta = std::move(theta);
+    b->h_prev = std::move(prev);
+    auto fail = [&](bbe_status code) {
+        bbe_destroy_batch(b);
+        return code;
+    };
+    bbe_status st = check_state(b);
+    Arena A;
+    if (st || (st = make_arena(b, A, s))) return fail(st);
+    void *d_rec = nullptr;
+    cudaError_t e = pool_alloc(&d_rec, rec.size() * sizeof(float), s);
+    if (e == cudaSuccess && t0) e = pool_alloc(&b->law_mem, 2 * size_t(b->n_races) * sizeof(float), s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_rec, rec.data(), rec.size() * sizeof(float), cudaMemcpyHostToDevice, s);
+    float *d_t0 = static_cast<float *>(b->law_mem), *d_inv = d_t0 ? d_t0 + b->n_races : nullptr;
+    if (e == cudaSuccess) {
+        repeat_records<<<unsigned((b->n_total + 255) / 256), 256, 0, s>>>(
+            Repeat{b->n_races, b->n_total, reps, n, n_rec, L, t0 ? 1.0f / T : 0.0f, R, static_cast<const float *>(d_rec),
+                   d_t0, d_inv, A});
+        e = cudaGetLastError();
+    }
+    if (d_rec) {
+        const cudaError_t f = cudaFreeAsync(d_rec, s);
+        if (e == cudaSuccess) e = f;
+    }
+    if (e != cudaSuccess) {
+        set_error(std::string("staging upload: ") + cudaGetErrorString(e));
+        return fail(BBE_ERR_CUDA);
+    }
+    b->dev = bbe::DevBatch{A.off, A.L, A.R, A.cr, A.d0, A.mu, A.sigma, A.rho, A.P, A.theta, A.prev, nullptr,
+                           b->n_races, b->n_total, race_id0, uint32_t(seed), uint32_t(seed >> 32), int32_t(dist)};
+    if (t0) {
+        b->h_t0 = *t0;
+        b->h_T.assign(size_t(n_rec), T);
+        b->dev.law = BBE_LAW_TIME;
+        b->dev.t0 = d_t0;
+        b->dev.invT = d_inv;
+    }
+    default_launch(b);
+    if ((st = build_items(b, s))) return fail(st);  // waits for the stream: rec and the batch are in place
+    *out = b;
+    return BBE_OK;
+}
 
 bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *race_off, const float *track_len,
                             const int64_t *rollouts, const float *pos, const float *mu, const float *sigma,
@@ -487,9 +734,11 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
         return BBE_ERR_ARG;
     }
     std::vector<int32_t> off(size_t(n_races) + 1);
-    bbe_status st = copy_in(off.data(), race_off, off.size() * sizeof(int32_t), s, "race_off");
+    bool pending = false;  // a copy from device memory is under way
+    bbe_status st = copy_in(off.data(), race_off, off.size() * sizeof(int32_t), s, "race_off", &pending);
     if (st) return st;
-    BBE_CUDA_TRY(cudaStreamSynchronize(s));
+    if (pending) BBE_CUDA_TRY(cudaStreamSynchronize(s));
+    pending = false;
     if (off[0] != 0) {
         set_error("race_off[0] != 0");
         return BBE_ERR_ARG;
@@ -510,8 +759,7 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
     const int32_t nt = off[n_races];
 
     auto b = new bbe_batch();
-    static std::atomic<uint64_t> next_serial{1};
-    b->serial = next_serial.fetch_add(1);
+    b->serial = g_next_serial.fetch_add(1);
     b->n_races = n_races;
     b->n_total = nt;
     b->max_n = max_n;
@@ -534,99 +782,35 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
         bbe_destroy_batch(b);  // frees whatever was allocated so far
         return code;
     };
-    if ((st = copy_in(b->h_L.data(), track_len, n_races * sizeof(float), s, "track_len")) ||
-        (st = copy_in(b->h_R.data(), rollouts, n_races * sizeof(int64_t), s, "rollouts")) ||
-        (st = copy_in(b->h_d0.data(), pos, nt * sizeof(float), s, "pos")) ||
-        (st = copy_in(b->h_mu.data(), mu, nt * sizeof(float), s, "mu")) ||
-        (st = copy_in(h_sigma.data(), sigma, nt * sizeof(float), s, "sigma")) ||
-        (st = copy_in(h_rho.data(), resp, nt * sizeof(float), s, "resp")) ||
-        (pref && (st = copy_in(h_P.data(), pref, nt * sizeof(float), s, "pref"))) ||
-        (theta && (st = copy_in(h_theta.data(), theta, nt * sizeof(float), s, "theta"))))
+    if ((st = copy_in(b->h_L.data(), track_len, n_races * sizeof(float), s, "track_len", &pending)) ||
+        (st = copy_in(b->h_R.data(), rollouts, n_races * sizeof(int64_t), s, "rollouts", &pending)) ||
+        (st = copy_in(b->h_d0.data(), pos, nt * sizeof(float), s, "pos", &pending)) ||
+        (st = copy_in(b->h_mu.data(), mu, nt * sizeof(float), s, "mu", &pending)) ||
+        (st = copy_in(h_sigma.data(), sigma, nt * sizeof(float), s, "sigma", &pending)) ||
+        (st = copy_in(h_rho.data(), resp, nt * sizeof(float), s, "resp", &pending)) ||
+        (pref && (st = copy_in(h_P.data(), pref, nt * sizeof(float), s, "pref", &pending))) ||
+        (theta && (st = copy_in(h_theta.data(), theta, nt * sizeof(float), s, "theta", &pending))))
         return fail(st);
     if (prev_step) {
         h_prev.resize(nt);
-        if ((st = copy_in(h_prev.data(), prev_step, nt * sizeof(float), s, "prev_step"))) return fail(st);
+        if ((st = copy_in(h_prev.data(), prev_step, nt * sizeof(float), s, "prev_step", &pending))) return fail(st);
     }
-    {
+    if (pending) {
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) {
             set_error(std::string("staging copies: ") + cudaGetErrorString(e));
             return fail(BBE_ERR_CUDA);
         }
     }
-    // validation (Section 3: S > 0, P in [0,1], positions on the track)
-    for (int r = 0; r < n_races; ++r) {
-        const float L = b->h_L[r];
-        if (!finite(L) || !(L > 0.0f)) {
-            set_error("track_len of race " + std::to_string(r) + " is not a positive finite number");
-            return fail(BBE_ERR_ARG);
-        }
-        if (b->h_R[r] < 1 || b->h_R[r] > INT32_MAX) {
-            set_error("rollouts of race " + std::to_string(r) + " outside 1..2^31-1");
-            return fail(BBE_ERR_ARG);
-        }
-        for (int i = off[r]; i < off[r + 1]; ++i) {
-            const float d = b->h_d0[i];
-            auto where = [&]() { return " (race " + std::to_string(r) + ", competitor " + std::to_string(i - off[r]) + ")"; };
-            if (!finite(d) || d < 0.0f) {
-                set_error("position must be finite and >= 0" + where());
-                return fail(BBE_ERR_ARG);
-            }
-            if (d >= L) {
-                set_error("competitor already finished (d >= L)" + where());
-                return fail(BBE_ERR_FINISHED);
-            }
-            if (!finite(b->h_mu[i]) || !(b->h_mu[i] > 0.0f) || !finite(h_sigma[i]) || !(h_sigma[i] >= 0.0f)) {
-                set_error("need finite mu > 0 and sigma >= 0" + where());
-                return fail(BBE_ERR_ARG);
-            }
-            if (!(h_rho[i] >= 0.0f && h_rho[i] <= 1.0f)) {
-                set_error("responsiveness rho outside [0, 1]" + where());
-                return fail(BBE_ERR_ARG);
-            }
-            if (!(h_P[i] > 0.0f && h_P[i] <= 1.0f)) {
-                set_error("preference P outside (0, 1]" + where());
-                return fail(BBE_ERR_ARG);
-            }
-            if (!finite(h_theta[i]) || !(h_theta[i] >= 0.0f)) {
-                set_error("theta must be finite and >= 0" + where());
-                return fail(BBE_ERR_ARG);
-            }
-            if (prev_step && (!finite(h_prev[i]) || !(h_prev[i] > 0.0f))) {
-                set_error("prev_step must be finite and > 0" + where());
-                return fail(BBE_ERR_ARG);
-            }
-        }
-    }
+    if ((st = check_state(b))) return fail(st);
     std::vector<int32_t> comp_race(nt);
     for (int r = 0; r < n_races; ++r)
         for (int i = off[r]; i < off[r + 1]; ++i) comp_race[i] = r;
 
-    // one device arena for the staged batch
-    size_t bytes = 0;
-    auto add = [&](size_t n) { bytes += (n + 255) / 256 * 256; };
-    add((n_races + 1) * 4); add(n_races * 4); add(n_races * 8); add(size_t(nt) * 4); add(n_races * 4);
-    for (int i = 0; i < 7; ++i) add(size_t(nt) * 4);
-    add((kGroups + 1 + size_t(n_races)) * 4);
-    cudaError_t e = cudaGetDevice(&b->device);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device);
-    if (e == cudaSuccess) e = pool_alloc(&b->arena, bytes, s);
-    if (e != cudaSuccess) {
-        set_error(std::string("device allocation: ") + cudaGetErrorString(e));
-        return fail(BBE_ERR_CUDA);
-    }
-    char *p = static_cast<char *>(b->arena);
-    int32_t *d_off = carve<int32_t>(p, n_races + 1);
-    float *d_L = carve<float>(p, n_races);
-    int64_t *d_R = carve<int64_t>(p, n_races);
-    int32_t *d_cr = carve<int32_t>(p, nt);
-    int32_t *d_ids = carve<int32_t>(p, n_races);
-    float *d_d0 = carve<float>(p, nt), *d_mu = carve<float>(p, nt), *d_sigma = carve<float>(p, nt);
-    float *d_rho = carve<float>(p, nt), *d_P = carve<float>(p, nt), *d_theta = carve<float>(p, nt);
-    float *d_prev = carve<float>(p, nt);
-    b->d_queue = carve<int32_t>(p, kGroups + 1 + size_t(n_races));
-    b->d_status = b->d_queue + kGroups;
-    b->d_next = b->d_status + 1;
+    Arena A;
+    if ((st = make_arena(b, A, s))) return fail(st);
+    const size_t bytes = A.bytes;
+    cudaError_t e = cudaSuccess;
     // A small batch's arena is assembled on the host in its own layout and goes up in one copy
     // (one transfer's overhead instead of one per array); a large one goes up array by array,
     // with no extra host pass over it.  The queue heads and status are reset before use.
@@ -635,13 +819,13 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
         const void *src;
         size_t n;
     };
-    std::vector<Up> ups = {{d_off, off.data(), off.size() * 4},       {d_L, b->h_L.data(), size_t(n_races) * 4},
-                           {d_R, b->h_R.data(), size_t(n_races) * 8}, {d_cr, comp_race.data(), size_t(nt) * 4},
-                           {d_d0, b->h_d0.data(), size_t(nt) * 4},   {d_mu, b->h_mu.data(), size_t(nt) * 4},
-                           {d_sigma, h_sigma.data(), size_t(nt) * 4}, {d_rho, h_rho.data(), size_t(nt) * 4},
-                           {d_P, h_P.data(), size_t(nt) * 4},         {d_theta, h_theta.data(), size_t(nt) * 4}};
-    if (prev_step) ups.push_back({d_prev, h_prev.data(), size_t(nt) * 4});
-    if (race_ids) ups.push_back({d_ids, b->h_race_ids.data(), size_t(n_races) * 4});
+    std::vector<Up> ups = {{A.off, off.data(), off.size() * 4},       {A.L, b->h_L.data(), size_t(n_races) * 4},
+                           {A.R, b->h_R.data(), size_t(n_races) * 8}, {A.cr, comp_race.data(), size_t(nt) * 4},
+                           {A.d0, b->h_d0.data(), size_t(nt) * 4},   {A.mu, b->h_mu.data(), size_t(nt) * 4},
+                           {A.sigma, h_sigma.data(), size_t(nt) * 4}, {A.rho, h_rho.data(), size_t(nt) * 4},
+                           {A.P, h_P.data(), size_t(nt) * 4},         {A.theta, h_theta.data(), size_t(nt) * 4}};
+    if (prev_step) ups.push_back({A.prev, h_prev.data(), size_t(nt) * 4});
+    if (race_ids) ups.push_back({A.ids, b->h_race_ids.data(), size_t(n_races) * 4});
     std::vector<char> img;
     if (bytes <= kOneCopyBytes) {
         img.assign(bytes, 0);
@@ -656,18 +840,11 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
             return fail(BBE_ERR_CUDA);
         }
     }
-    e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        set_error(std::string("staging upload: ") + cudaGetErrorString(e));
-        return fail(BBE_ERR_CUDA);
-    }
-    b->dev = bbe::DevBatch{d_off,   d_L,      d_R,   d_cr, d_d0, d_mu, d_sigma, d_rho, d_P, d_theta,
-                           prev_step ? d_prev : nullptr, race_ids ? d_ids : nullptr, n_races, nt, race_id0,
+    b->dev = bbe::DevBatch{A.off,   A.L,      A.R,   A.cr, A.d0, A.mu, A.sigma, A.rho, A.P, A.theta,
+                           prev_step ? A.prev : nullptr, race_ids ? A.ids : nullptr, n_races, nt, race_id0,
                            uint32_t(seed), uint32_t(seed >> 32), int32_t(dist)};
-    b->cfg = bbe_launch_cfg{kDefaultWarpsPerBlock, kDefaultBlocksPerSm, kDefaultRolloutsPerLane, BBE_MAX_STEPS_DEFAULT, 0};
-    for (int g = 0; g < kGroups; ++g)
-        b->resident[g] = bbe::rollout_resident_blocks(b->dist, kSlots[g], 32 * kDefaultWarpsPerBlock);
-    if ((st = build_items(b, s))) return fail(st);
+    default_launch(b);
+    if ((st = build_items(b, s))) return fail(st);  // waits for the stream: all uploads are in place
     *out = b;
     return BBE_OK;
 }
@@ -678,6 +855,7 @@ bbe_status bbe::set_first_rollouts(bbe_batch *b, const int64_t *k0)
         set_error("batch or k0 is NULL");
         return BBE_ERR_ARG;
     }
+    unfold(b);
     for (int r = 0; r < b->n_races; ++r) {
         if (k0[r] < 0 || k0[r] + b->h_R[r] > INT32_MAX) {
             set_error("first rollout index out of range");
@@ -784,6 +962,7 @@ bbe_status run_place_mode(bbe_batch *b, int32_t places, int32_t *place_counts, i
 // per-race first entries of the order tally tables for `places` (n_r ^ min(places, n_r) entries)
 void order_layout(const bbe_batch *b, int32_t places, std::vector<int64_t> &off)
 {
+    bbe::unfold(b);
     off.assign(size_t(b->n_races) + 1, 0);
     for (int r = 0; r < b->n_races; ++r) {
         const int n = b->h_off[r + 1] - b->h_off[r];
@@ -810,6 +989,7 @@ uint64_t ordered_tuples(int n, int K)
 // at least 2; false (with the error set) for a race whose order keys do not fit in 64 bits
 bool hist_layout(const bbe_batch *b, int32_t places, std::vector<int64_t> &off)
 {
+    bbe::unfold(b);
     off.assign(size_t(b->n_races) + 1, 0);
     for (int r = 0; r < b->n_races; ++r) {
         const int n = b->h_off[r + 1] - b->h_off[r];
@@ -1035,6 +1215,7 @@ bbe_status bbe_batch_set_law(bbe_batch *b, bbe_law law, const float *elapsed, co
         return BBE_ERR_ARG;
     }
     cudaStream_t s = as_stream(cuda_stream);
+    bbe::unfold(b);
     if (law == BBE_LAW_POSITION) {
         b->dev.law = BBE_LAW_POSITION;
         b->h_t0.clear();
@@ -1167,6 +1348,7 @@ bbe_status bbe_batch_autotune(bbe_batch *b, int32_t *win_counts, double budget_m
         return BBE_ERR_ARG;
     }
     cudaStream_t s = as_stream(cuda_stream);
+    bbe::unfold(b);
     const bbe_launch_cfg start = b->cfg;
     int8_t start_tab[BBE_MAX_COMPETITORS + 1];
     std::memcpy(start_tab, b->slots_by_n, sizeof(start_tab));
@@ -1332,7 +1514,7 @@ bbe_status bbe_batch_info(const bbe_batch *b, int32_t *n_races, int64_t *n_compe
     }
     if (n_races) *n_races = b->n_races;
     if (n_competitors) *n_competitors = b->n_total;
-    if (total_rollouts) *total_rollouts = std::accumulate(b->h_R.begin(), b->h_R.end(), int64_t(0));
+    if (total_rollouts) *total_rollouts = std::accumulate(b->h_R.begin(), b->h_R.end(), int64_t(0)) * b->reps;
     if (max_competitors) *max_competitors = b->max_n;
     return BBE_OK;
 }

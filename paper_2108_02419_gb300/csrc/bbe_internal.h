@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <type_traits>
 #include <utility>
@@ -177,7 +178,11 @@ struct bbe_batch {
     int32_t dist = 0;
     uint32_t race_id0 = 0;
 
-    // host copies (scheduling, cost estimates, range checks and sub-batches)
+    // host copies (scheduling, cost estimates, range checks and sub-batches), one record per race, or
+    // one per `reps` consecutive races that differ in their stream ids alone (bbe_snapshot_batch);
+    // bbe::unfold makes it one per race for whoever needs that
+    int32_t reps = 1;
+    std::mutex unfold_mu;
     std::vector<int32_t> h_off;
     std::vector<float> h_L;
     std::vector<int64_t> h_R;
@@ -245,6 +250,15 @@ bbe_status stage_batch(bbe_batch **out, int32_t n_races, const int32_t *race_off
 // k0[r] + R[r] <= 2^31 - 1).  The counts of such a batch added to those of rollouts
 // 0 .. k0[r] - 1 equal the counts of one batch of k0[r] + R[r] rollouts.
 bbe_status set_first_rollouts(bbe_batch *b, const int64_t *k0);
+// A batch of n_rec x reps races of n competitors each: race r has record r / reps (host arrays, n_rec or
+// n_rec x n entries), track length L, R rollouts and stream id race_id0 + r.  t0: elapsed steps per
+// record under the time law with expected duration T, or null for the position law.
+bbe_status stage_repeated(bbe_batch **out, int32_t n_rec, int32_t reps, int32_t n, float L, int64_t R,
+                          std::vector<float> d0, std::vector<float> mu, std::vector<float> sigma, std::vector<float> rho,
+                          std::vector<float> P, std::vector<float> theta, std::vector<float> prev, uint64_t seed,
+                          bbe_dist dist, uint32_t race_id0, const std::vector<float> *t0, float T, cudaStream_t s);
+// The host copies of such a batch, one record per race from here on.
+void unfold(const bbe_batch *b);
 // Record that work just enqueued on `s` reads the batch (see bbe_batch::uses).
 cudaError_t note_use(const bbe_batch *b, cudaStream_t s);
 }  // namespace bbe

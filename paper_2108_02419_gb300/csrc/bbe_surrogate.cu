@@ -2275,6 +2275,7 @@ bbe_status bbe_surrogate_grad(bbe_surrogate *s, const bbe_batch *b, const float 
         bbe::set_error("the surrogate takes position-law batches only (its inputs carry no elapsed time)");
         return BBE_ERR_UNSUPPORTED;
     }
+    bbe::unfold(b);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     bbe_status e;
     if ((e = ensure_attrs())) return e;
@@ -2303,6 +2304,7 @@ bbe_status bbe_surrogate_train(bbe_surrogate *s, const bbe_batch *b, const float
         bbe::set_error("the surrogate takes position-law batches only (its inputs carry no elapsed time)");
         return BBE_ERR_UNSUPPORTED;
     }
+    bbe::unfold(b);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     bbe_status e;
     if ((e = ensure_attrs())) return e;
@@ -2366,6 +2368,7 @@ bbe_status bbe_surrogate_forward(bbe_surrogate *s, const bbe_batch *b, float *pr
         bbe::set_error("the surrogate takes position-law batches only (its inputs carry no elapsed time)");
         return BBE_ERR_UNSUPPORTED;
     }
+    bbe::unfold(b);
     std::vector<int32_t> order(b->n_races);
     std::iota(order.begin(), order.end(), 0);
     return forward_all(s, b, order, probs, reinterpret_cast<cudaStream_t>(cuda_stream));
@@ -2382,6 +2385,7 @@ bbe_status bbe_surrogate_infer(bbe_surrogate *s, const bbe_batch *b, float *prob
         bbe::set_error("the surrogate takes position-law batches only (its inputs carry no elapsed time)");
         return BBE_ERR_UNSUPPORTED;
     }
+    bbe::unfold(b);
     if (!s->ranges.valid) {
         bbe::set_error("bbe_surrogate_infer: the network has no training ranges (train or load it first)");
         return BBE_ERR_RANGE;

@@ -228,6 +228,7 @@ bbe_status bbe_snapshot_batch(bbe_batch **out, const bbe_batch *src, int32_t rac
     }
     *out = nullptr;
     cudaStream_t s = as_stream(cuda_stream);
+    bbe::unfold(src);
     const int off = src->h_off[race];
     const int n = src->h_off[race + 1] - off;
     int32_t steps = 0;
@@ -259,49 +260,32 @@ bbe_status bbe_snapshot_batch(bbe_batch **out, const bbe_batch *src, int32_t rac
         bbe::set_error("bbe_snapshot_batch: no open snapshot, or too many races");
         return BBE_ERR_RANGE;
     }
-    const size_t nr = size_t(n_races);
-    std::vector<int32_t> roff(nr + 1, 0);
-    std::vector<int32_t> ids(nr, 0);
-    std::vector<float> Ls(nr, L);
-    std::vector<int64_t> R(nr, dry_runs);
-    const size_t nt = size_t(n_races) * n;
-    std::vector<float> d0(nt), mu(nt), sg(nt), rho(nt), P(nt), th(nt), pv(nt);
+    // one record per snapshot; its bettors' races differ in their stream ids alone
+    const size_t nt = times.size() * size_t(n);
+    std::vector<float> d0(nt), mu(nt), sg(nt), rho(nt), P(nt), th(nt), pv(nt), el(times.size());
     size_t i = 0;
     for (size_t si = 0; si < times.size(); ++si) {
         const int ts = times[si];
-        for (int bt = 0; bt < bettors; ++bt) {
-            const size_t rr = si * size_t(bettors) + size_t(bt);
-            roff[rr + 1] = roff[rr] + n;
-            ids[rr] = int32_t(race_id0 + uint32_t(rr));
-            for (int c = 0; c < n; ++c, ++i) {
-                const int ci = off + c;
-                d0[i] = ts == 0 ? src->h_d0[ci] : pos[size_t(ts - 1) * n + c];
-                mu[i] = src->h_mu[ci];
-                sg[i] = src->h_sigma[ci];
-                rho[i] = src->h_rho[ci];
-                P[i] = src->h_P[ci];
-                th[i] = src->h_theta[ci];
-                pv[i] = ts > 0 ? stp[size_t(ts - 1) * n + c]
-                               : (src->h_prev.empty() ? src->h_mu[ci] * src->h_P[ci] : src->h_prev[ci]);
-            }
+        for (int c = 0; c < n; ++c, ++i) {
+            const int ci = off + c;
+            d0[i] = ts == 0 ? src->h_d0[ci] : pos[size_t(ts - 1) * n + c];
+            mu[i] = src->h_mu[ci];
+            sg[i] = src->h_sigma[ci];
+            rho[i] = src->h_rho[ci];
+            P[i] = src->h_P[ci];
+            th[i] = src->h_theta[ci];
+            pv[i] = ts > 0 ? stp[size_t(ts - 1) * n + c]
+                           : (src->h_prev.empty() ? src->h_mu[ci] * src->h_P[ci] : src->h_prev[ci]);
         }
-    }
-    bbe_status e = bbe::stage_batch(out, int32_t(n_races), roff.data(), Ls.data(), R.data(), d0.data(), mu.data(),
-                                    sg.data(), rho.data(), P.data(), th.data(), pv.data(), src->seed,
-                                    bbe_dist(src->dist), race_id0, ids.data(), s);
-    if (e) return e;
-    if (src->dev.law == BBE_LAW_TIME) {
         // a snapshot taken ts steps into the actual race has run t0 + ts steps; same horizon
-        std::vector<float> el(nr), hz(nr, src->h_T[size_t(race)]);
-        for (size_t si = 0; si < times.size(); ++si)
-            for (int bt = 0; bt < bettors; ++bt)
-                el[si * size_t(bettors) + size_t(bt)] = src->h_t0[size_t(race)] + float(times[si]);
-        if ((e = bbe_batch_set_law(*out, BBE_LAW_TIME, el.data(), hz.data(), s))) {
-            bbe_destroy_batch(*out);
-            *out = nullptr;
-            return e;
-        }
+        if (src->dev.law == BBE_LAW_TIME) el[si] = src->h_t0[size_t(race)] + float(ts);
     }
+    const bool time_law = src->dev.law == BBE_LAW_TIME;
+    const bbe_status e = bbe::stage_repeated(
+        out, int32_t(times.size()), bettors, n, L, dry_runs, std::move(d0), std::move(mu), std::move(sg), std::move(rho),
+        std::move(P), std::move(th), std::move(pv), src->seed, bbe_dist(src->dist), race_id0, time_law ? &el : nullptr,
+        time_law ? src->h_T[size_t(race)] : 0.0f, s);
+    if (e) return e;
     *n_snapshots = int32_t(times.size());
     return BBE_OK;
 }
