@@ -28,17 +28,17 @@
 // (contender_line); they take the slots, so a warp has room for more segments.  A work item is a
 // ticket for some of a race's rollouts, and the warp takes as many as its segments can share.
 //
-// Finishing.  A ballot finds the steps with finishers; each finisher offers the key
-// (within-step crossing time tau = (L - d) / S, slot) to its segment's minimum in shared
-// memory, which gives the least tau and, on equal tau, the lowest competitor index.  Wins are
-// tallied per competitor in shared memory and reach the global counts once per work item.
-// Place mode records each crossing with its key (sub-step, tau, slot) and places a block's
-// crossings at the block's end; a segment whose K-th place is filled ends its rollout, and its
-// places and order are tallied when it restarts.
-//
-// Loop bookkeeping.  After a block without a finish or a step-limit cut-off nothing can have
-// changed which slots run, so the warp's reduction of restart and liveness flags runs only after
-// blocks with one; a warp-uniform count-down rules out the step limit until a block could reach it.
+// Finishing.  A rollout that ends waits for the block's end in any case, and what its slots do until
+// then counts for nobody.  So the steps know nothing of the line: one vote a block finds the blocks
+// with crossings (positions only grow), and the positions published in the block say which step each
+// was.  The least key (step, within-step crossing time tau = (L - d) / S, slot) of a segment is the
+// first finisher: the least tau and, on equal tau, the lowest competitor index.  Wins are tallied per
+// competitor in shared memory and reach the global counts once per work item.  Place mode places a
+// block's crossings in key order until the K-th place is filled.  The step limit is looked at in the
+// same place, and a warp-uniform count-down rules it out until a block could reach it.  (With the
+// finish found within its step, a vote a step and a copy of the step for blocks near the limit: 4096
+// spread races of 20 52.0 instead of 50.0 ms, 10^4 uneven ones 80.3 instead of 78.4, 700 bunched of 13
+// 15.5 instead of 14.7, places 19.5 instead of 18.3.)
 //
 // The arithmetic is the pinned binary32 round-to-nearest sequence of include/bbe.h (explicit
 // intrinsics, file compiled with --fmad=false), so the counts are bit-identical to any
@@ -59,32 +59,37 @@ namespace win {
 
 constexpr unsigned kAll = 0xffffffffu;
 constexpr unsigned long long kNoKey = ~0ull;
-constexpr uint8_t kNoSub = 255;
+constexpr int kPlaced = 128;           // place mode: a segment's K places are filled, at this step of the block
+constexpr unsigned kNone = ~0u;       // win mode: a segment without a finish, ..
+constexpr unsigned kCut = kNone - 1u;  // .. and one whose rollout has run its last step without one
 
-template <int V>
+template <int V, int MODE>
 struct WinStage {
     static constexpr int NS = 32 * V;   // slots per warp
     static constexpr int ROW = NS + 2;  // entries per position row: slots, the sentinel, padding to 16 bytes
-    float2 pos[2][ROW];                 // (d, previous step) per slot, one row per step parity
+    float2 pos[4][ROW];                 // (d, previous step) per slot, one row per step of a block
     float4 pq[32];                      // per competitor: (mu, sigma, P, theta)
     float kr[32];                       // per competitor: kappa (2 rho - 1)
+    unsigned pha[32];                   // per competitor: StreamWords::a, the same for all rollouts
     float d0[32], prev0[32];            // per competitor: start state of every rollout
     uint4 ph[NS];                       // per slot: the current rollout's Philox constants (StreamWords)
-    unsigned pha[NS];
     unsigned segk[NS];                  // by segment base: rollout index handed to a restart
-    int wins[32];                       // wins per competitor in the current work item
-    unsigned long long key[NS];         // by segment base: least crossing key of the block (win mode)
-    float2 fcross[NS];                  // place mode: (d, S) of each slot's crossing in the block
-    // Rank order (ascending position, then slot).  A segment of n slots has n + 1 entries of `order`,
-    // the slots by rank and the sentinel behind them, so the entry after a slot's own is its
-    // successor's; `at` is a slot's own entry and `flag` marks the entries that swap with the next.
+    int wins[MODE == 0 ? 32 : 1];       // wins per competitor in the current work item
+    // by segment base; win mode: the block's least (step, tau) and the first slot that has it; place
+    // mode: the least crossing key not yet placed
+    union {
+        unsigned win[2][NS];
+        unsigned long long place[NS];
+    } key;
+    // Rank order (ascending position, then slot).  A segment of n slots with first slot sb has the
+    // entries of `order` from 1 + 2 sb on: its slots by rank and the sentinel behind them, so the entry
+    // after a slot's own is its successor's (order[0] and flag[0] are nobody's); `at` is a slot's own
+    // entry and `flag` marks the entries that swap with the next.
     uint8_t order[2 * NS + 4], flag[2 * NS + 4];
     uint8_t at[NS];
-    uint8_t fsub[NS];                   // place mode: sub-step of each slot's crossing in the block, or kNoSub
-    uint8_t base[NS], rbase[NS];        // first slot and first order entry of each slot's segment
+    uint8_t base[NS];                   // first slot of each slot's segment
     uint8_t rank0[32], byrank0[32];     // start rank of competitor c; competitor at start rank r
     uint8_t comp[32];                   // the race's index of competitor c (its stream and its count)
-    unsigned next_k;                    // next rollout index of the work item
 };
 
 __device__ __forceinline__ float warp_min(float v)
@@ -203,12 +208,12 @@ __device__ __forceinline__ void draw_block(const uint4 &q, uint32_t a, uint32_t 
 }
 
 // Registers per thread.  Win counts: 80 for two slots per lane (6 resident 4-warp blocks per SM) and
-// 56 for one; with 72 and 48 (7 and 10 blocks) a pass over 4096 races of 20 takes 57.1 instead of
-// 54.7 ms and one small race 59 instead of 56 us.  Place mode spills nothing at 72, and fewer warps
+// 64 for one; with 72 and 56 (7 and 9 blocks) a pass over 4096 races of 20 takes 57.1 instead of
+// 54.7 ms and one small race, run in that layout, 42 instead of 37 us.  Place mode spills nothing at 72, and fewer warps
 // cost it 1 %.  Three and four slots per lane read their parameters from shared memory.
 template <int V, int MODE>
 struct WinRegs {
-    static constexpr int value = V == 1 ? (MODE == 0 ? 56 : 48) : (V == 2 ? (MODE == 0 ? 80 : 72) : 80);
+    static constexpr int value = V == 1 ? (MODE == 0 ? 64 : 48) : (V == 2 ? (MODE == 0 ? 80 : 72) : 80);
 };
 // Parameters read from shared memory each step instead of held in registers.
 template <int V>
@@ -224,7 +229,7 @@ template <int DIST, int V, int LAW, int MODE>
 __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(RolloutLaunch l)
 {
     constexpr bool PS = WinLean<V>::value;
-    using Stage = WinStage<V>;
+    using Stage = WinStage<V, MODE>;
     constexpr int NS = Stage::NS;
     constexpr int ROWB = Stage::ROW * int(sizeof(float2));
     constexpr int kSent = NS * int(sizeof(float2));  // byte offset of the sentinel (+inf: no one in front)
@@ -232,22 +237,19 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
     Stage &st = reinterpret_cast<Stage *>(win_smem)[threadIdx.x >> 5];
     char *const posb = reinterpret_cast<char *>(&st.pos[0][0]);
     // place mode, per warp after all the stages: the finisher of each place (by segment base +
-    // place), the places filled and the sub-step of the K-th place (by segment base), then the
-    // work item's [competitor][place] table
-    uint8_t *pl_ord = nullptr, *pl_n = nullptr, *pl_kj = nullptr;
+    // place), the places filled (by segment base), then the work item's [competitor][place] table
+    uint8_t *pl_ord = nullptr, *pl_n = nullptr;
     int *pl_cnt = nullptr;
     if constexpr (MODE == 1) {
         pl_cnt = reinterpret_cast<int *>(win_smem + (blockDim.x >> 5) * sizeof(Stage)) +
-                 (threadIdx.x >> 5) * (3 * NS / 4 + l.place_cells);
+                 (threadIdx.x >> 5) * (NS / 2 + l.place_cells);
         pl_ord = reinterpret_cast<uint8_t *>(pl_cnt + l.place_cells);
         pl_n = pl_ord + NS;
-        pl_kj = pl_ord + 2 * NS;
     }
     const DevBatch &b = l.b;
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
-        st.pos[0][NS] = make_float2(INFINITY, INFINITY);
-        st.pos[1][NS] = make_float2(INFINITY, INFINITY);
+        for (int j = 0; j < 4; ++j) st.pos[j][NS] = make_float2(INFINITY, INFINITY);
     }
     for (;;) {
         int it = 0;
@@ -263,6 +265,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         const float invL = __fdiv_rn(1.0f, L);
         const float t0r = LAW == BBE_LAW_TIME ? b.t0[r] : 0.0f;     // time law: elapsed steps
         const float invTr = LAW == BBE_LAW_TIME ? b.invT[r] : 0.0f;  // time law: 1 / expected duration
+        const uint32_t rid = b.race_ids ? uint32_t(b.race_ids[r]) : b.race_id0 + uint32_t(r);
         // a ticket: nothing to do once the race's rollouts have all been taken
         const int64_t Rr = b.R[r];
         if (l.next != nullptr) {
@@ -334,12 +337,18 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             st.d0[c] = my_d0;
             st.prev0[c] = my_pv;
             st.comp[c] = uint8_t(lane);
-            st.wins[c] = 0;
+            if constexpr (MODE == 0) st.wins[c] = 0;
+            st.pha[c] = stream_words(0u, uint32_t(lane), rid, l.round_key).a;
             st.rank0[c] = uint8_t(rank);
             st.byrank0[BBE_INDEX(rank, 32, l.status)] = uint8_t(c);
         }
         for (int i = lane; i < NS; i += 32) {
-            st.key[i] = kNoKey;
+            if constexpr (MODE == 1) {
+                st.key.place[i] = kNoKey;
+                pl_n[i] = 0;
+            } else {
+                st.key.win[0][i] = st.key.win[1][i] = kNone;
+            }
             st.order[2 * i] = st.order[2 * i + 1] = uint8_t(NS);
             st.flag[2 * i] = st.flag[2 * i + 1] = 0;
         }
@@ -349,43 +358,32 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         }
         const int K = MODE == 1 ? min(l.places, n) : 1;  // places run per rollout
         if constexpr (MODE == 1) {
-            for (int i = lane; i < NS; i += 32) {
-                pl_n[i] = 0;
-                st.fsub[i] = kNoSub;
-            }
             for (int i = lane; i < n * K; i += 32) pl_cnt[i] = 0;
         }
-        if (lane == 0) st.next_k = k_begin + unsigned(nseg);
         __syncwarp();
 
-        const uint32_t rid = b.race_ids ? uint32_t(b.race_ids[r]) : b.race_id0 + uint32_t(r);
         // unsigned: rollout indices stay below 2^31 + 2^7
         const unsigned kend = k_begin + k_count;
+        unsigned next_k = k_begin + unsigned(nseg);  // warp-uniform: the next segment that is free takes it
 
         // per slot: segment base, competitor parameters, state, front address, rollout, block
         int fo[V];
-        unsigned blk[V];
+        unsigned blk[V], pha[V];
         float mu[V], sg[V], P[V], th[V], kr[V], d[V], pv[V];
         const float4 *pqa[V];  // register-lean variant: this slot's (mu, sigma, P, theta)
         const float *kra[V];   // register-lean variant: this slot's kappa (2 rho - 1)
         // a slot that runs no rollout has no position (NaN): it is never out of order, never over
         // the line, and stays so without a test in the step
-        bool pend[V], cut[V];  // rollout ended, to restart; stopped at max_steps
+        bool pend[V];  // rollout ended, to restart
         auto alive = [&](int v) { return d[v] == d[v]; };
         auto base = [&](int v) { return int(st.base[32 * v + lane]); };
         // slot's stream for rollout k (competitor c of the advanced ones)
         auto set_stream = [&](int slot, unsigned k, int c) {
             const StreamWords q = stream_words(k, uint32_t(st.comp[c]), rid, l.round_key);
             st.ph[slot] = make_uint4(q.d, q.e, q.f, q.g);
-            st.pha[slot] = q.a;
         };
         const float kDead = __int_as_float(0x7fffffff);
-        auto stop = [&](int v) {  // this slot's rollout is over
-            d[v] = kDead;
-            fo[v] = kSent;
-        };
         unsigned long long steps = 0;
-        bool blk_fin = false;  // warp-uniform: some slot crossed the line in this block (a finish)
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const int slot = 32 * v + lane;
@@ -396,17 +394,16 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             const unsigned k = k_begin + unsigned(seg);
             const bool run = used && k < kend;
             st.base[slot] = uint8_t(sb);
-            const int rb = 1 + (used ? seg * (n + 1) : 0);  // order[0] and flag[0] are nobody's
-            st.rbase[slot] = uint8_t(rb);
+            const int rb = 1 + 2 * sb;
             st.at[slot] = uint8_t(rb);
             set_stream(slot, k, c);
             pend[v] = false;
-            cut[v] = false;
             blk[v] = 0;
             if constexpr (PS) {
                 pqa[v] = &st.pq[c];
                 kra[v] = &st.kr[c];
             } else {
+                pha[v] = st.pha[c];
                 const float4 q = st.pq[c];
                 mu[v] = q.x;
                 sg[v] = q.y;
@@ -441,7 +438,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     rk += dj < d[v] || (dj == d[v] && j < slot) ? 1 : 0;
                 }
                 if (alive(v)) {
-                    const int a = BBE_INDEX(int(st.rbase[slot]) + rk, 2 * NS + 3, l.status);
+                    const int a = BBE_INDEX(1 + 2 * sb + rk, 2 * NS + 3, l.status);
                     st.order[a] = uint8_t(slot);
                     st.at[slot] = uint8_t(a);
                 }
@@ -509,80 +506,124 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             if (__any_sync(kAll, again)) full_sort(pb, fd, fp);
         };
 
-        // Place mode, the end of a Philox block in which some slot crossed the line or may have
-        // reached max_steps: the block's crossings of each segment take the next places one at
-        // a time in key order (sub-step, tau, slot), and a segment whose K-th place is filled
-        // ends its rollout (its places and order are tallied when it restarts); a rollout
-        // stopped at max_steps that did not end earlier counts for nobody.  Ending at the
-        // block's end costs nothing: a segment whose rollout ended waits for the next block in
-        // any case, and its slots record no further crossings (d < L fails past the line).
-        // (Measured slower for win counts, which end their rollouts within the step.)
-        auto block_end = [&]() {
-            __syncwarp();
-            {
-                unsigned long long fk[V];
-                int sb[V];
-                bool more = false;
+        // Steps of a Philox block past a crossing, or past the step limit, change nothing that counts (the
+        // rollout ends with the block in any case), so crossings are looked for once a block: positions
+        // only grow, and the block's four rows say which step it was.  (d, S) of that step, for a slot that
+        // has crossed in this block:
+        auto crossing = [&](int v, float &dc, float &Sc) {
+            const int slot = 32 * v + lane;
+            const int J = (st.pos[1][slot].x < L ? 1 : 0) + (st.pos[2][slot].x < L ? 1 : 0) + (st.pos[3][slot].x < L ? 1 : 0);
+            dc = st.pos[J][slot].x;
+            Sc = J < 3 ? st.pos[J + 1][slot].y : pv[v];
+            return J;
+        };
+
+        // Win mode, the end of a block with a crossing (or, chk, one in which a rollout may have run its
+        // last step): the least key (step, tau) of each segment, then the least slot that has it.  tau =
+        // (L - d) / S is in [0, 2], so its bit pattern less one orders like its value and fits in 30 bits.
+        auto win_end = [&](bool chk) {
+            unsigned mine[V], kw[V];
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const int slot = 32 * v + lane;
-                    sb[v] = base(v);
-                    const unsigned sub = st.fsub[slot];
-                    fk[v] = kNoKey;
-                    if (sub != kNoSub) {
-                        const float2 c = st.fcross[slot];
-                        const float tau = __fdiv_rn(__fsub_rn(L, c.x), c.y);
-                        fk[v] = (static_cast<unsigned long long>(sub) << 40) |
+            for (int v = 0; v < V; ++v) {
+                mine[v] = kNone;
+                if (d[v] >= L) {
+                    float dc, Sc;
+                    const int J = crossing(v, dc, Sc);
+                    if (!chk || int(blk[v]) * 4 - 4 + J < limit) {
+                        const unsigned tau = __float_as_uint(__fdiv_rn(__fsub_rn(L, dc), Sc));
+                        mine[v] = (unsigned(J) << 30) | (max(tau, 1u) - 1u);
+                        atomicMin(&st.key.win[0][base(v)], mine[v]);
+                    }
+                }
+                if (chk && alive(v) && int(blk[v]) * 4 >= limit) atomicMin(&st.key.win[0][base(v)], kCut);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                kw[v] = alive(v) ? st.key.win[0][base(v)] : kNone;
+                pend[v] = kw[v] != kNone;
+                if (pend[v] && mine[v] == kw[v]) atomicMin(&st.key.win[1][base(v)], unsigned(32 * v + lane));
+            }
+            __syncwarp();
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int slot = 32 * v + lane;
+                if (!pend[v] || slot != base(v)) continue;
+                if (kw[v] == kCut) {
+                    if (limit < l.max_steps) redo = true;
+                    else atomicOr(l.status, kStatusStepLimit);
+                    steps += (unsigned long long)l.max_steps;
+                } else {
+                    atomicAdd(&st.wins[BBE_INDEX(int(st.key.win[1][slot]) - slot, 32, l.status)], 1);
+                    steps += (unsigned long long)(blk[v] * 4u - 3u + (kw[v] >> 30));
+                }
+                st.key.win[0][slot] = st.key.win[1][slot] = kNone;
+            }
+        };
+
+        // Place mode, the same: the block's crossings of each segment take the next places one at a
+        // time in key order (step, tau, slot), and a segment whose K-th place is filled ends its
+        // rollout; one stopped at max_steps that did not end earlier counts for nobody.
+        auto place_end = [&](bool chk) {
+            unsigned long long fk[V];
+            int sb[V];
+            bool more = false;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int slot = 32 * v + lane;
+                sb[v] = base(v);
+                fk[v] = kNoKey;
+                if (d[v] >= L && st.pos[0][slot].x < L) {
+                    float dc, Sc;
+                    const int J = crossing(v, dc, Sc);
+                    if (!chk || int(blk[v]) * 4 - 4 + J < limit) {
+                        const float tau = __fdiv_rn(__fsub_rn(L, dc), Sc);
+                        fk[v] = (static_cast<unsigned long long>(J) << 40) |
                                 (static_cast<unsigned long long>(__float_as_uint(tau)) << 8) | unsigned(slot);
-                        st.fsub[slot] = kNoSub;
                         more = true;
                     }
                 }
-                // one crossing per segment per round; a segment has at most n of them
-                for (int round = 0; round < NS && __any_sync(kAll, more); ++round) {
+            }
+            // one crossing per segment per round; a segment has at most n of them
+            for (int round = 0; round < NS && __any_sync(kAll, more); ++round) {
 #pragma unroll
-                    for (int v = 0; v < V; ++v)
-                        if (fk[v] != kNoKey) atomicMin(&st.key[sb[v]], fk[v]);
-                    __syncwarp();
-                    bool won[V];
+                for (int v = 0; v < V; ++v)
+                    if (fk[v] != kNoKey) atomicMin(&st.key.place[sb[v]], fk[v]);
+                __syncwarp();
+                bool won[V];
 #pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        won[v] = fk[v] != kNoKey && st.key[sb[v]] == fk[v];
-                        if (won[v]) {
-                            const int p = BBE_INDEX(int(pl_n[sb[v]]), n, l.status);
-                            pl_ord[sb[v] + p] = uint8_t(32 * v + lane - sb[v]);
-                            pl_n[sb[v]] = uint8_t(p + 1);
-                            if (p == K - 1) pl_kj[sb[v]] = uint8_t(fk[v] >> 40);
-                        }
+                for (int v = 0; v < V; ++v) {
+                    won[v] = fk[v] != kNoKey && st.key.place[sb[v]] == fk[v];
+                    if (won[v] && pl_n[sb[v]] < K) {
+                        const int p = BBE_INDEX(int(pl_n[sb[v]]), K, l.status);
+                        pl_ord[sb[v] + p] = uint8_t(32 * v + lane - sb[v]);
+                        pl_n[sb[v]] = uint8_t(p + 1 < K ? p + 1 : kPlaced + int(fk[v] >> 40));
                     }
-                    __syncwarp();
-                    more = false;
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        if (fk[v] != kNoKey) st.key[sb[v]] = kNoKey;
-                        if (won[v]) fk[v] = kNoKey;
-                        more |= fk[v] != kNoKey;
-                    }
-                    __syncwarp();
                 }
+                __syncwarp();
+                more = false;
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    if (fk[v] != kNoKey) st.key.place[sb[v]] = kNoKey;
+                    if (won[v]) fk[v] = kNoKey;
+                    more |= fk[v] != kNoKey;
+                }
+                __syncwarp();
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                if (!alive(v) && !cut[v]) continue;
-                const int slot = 32 * v + lane, sb = base(v);
-                const int jend = pl_n[sb] >= K ? pl_kj[sb] : -1;  // sub-step of the K-th place
-                if (jend >= 0) {
-                    if (slot == sb) steps += (unsigned long long)(blk[v] * 4u + unsigned(jend) + 1u);
+                if (!alive(v)) continue;
+                const int slot = 32 * v + lane;
+                const unsigned filled = pl_n[sb[v]];
+                if (filled >= kPlaced) {
+                    if (slot == sb[v]) steps += (unsigned long long)(blk[v] * 4u - 3u + filled - kPlaced);
                     pend[v] = true;
-                } else if (cut[v]) {
-                    if (slot == sb) steps += (unsigned long long)l.max_steps;
+                } else if (chk && int(blk[v]) * 4 >= limit) {
+                    if (slot == sb[v]) steps += (unsigned long long)l.max_steps;
                     atomicOr(l.status, kStatusStepLimit);
                     pend[v] = true;
                 }
-                if (pend[v]) stop(v);
-                cut[v] = false;
             }
-            __syncwarp();
         };
 
         // Place mode, at a block boundary: the segments that completed a rollout (K places filled;
@@ -594,7 +635,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 const int sb = base(v);
-                if (!pend[v] || pl_n[sb] < K) continue;
+                if (!pend[v] || pl_n[sb] < kPlaced) continue;
                 const int c = 32 * v + lane - sb;  // this slot's competitor
                 if (c < K) atomicAdd(&pl_cnt[BBE_INDEX(pl_ord[sb + c] * K + c, n * K, l.status)], 1);
                 if (c == 0 && (l.orders != nullptr || l.hist_keys != nullptr)) {
@@ -622,31 +663,11 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             __syncwarp();
         };
 
-        // One step of every slot: sub-step j0 + J of the Philox block (its normal is z[v][J]); CHK
-        // when some segment may reach its limit within the block.
+        // One step of every slot: step j0 + J of the Philox block, with the normal z[v][J].
         int j0 = 0;
-        auto step = [&](auto Jc, auto CHKc, const float (&z)[V][4]) {
-            const int J = Jc;  // a compile-time constant, but for the rare checked block
-            constexpr bool CHK = decltype(CHKc)::value;
-            const int BO = (J & 1) * ROWB;
-            if constexpr (CHK) {
-                // a rollout reaching step max_steps stops there and counts for nobody (in place
-                // mode unless it ended earlier in the block, decided at the block's end)
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    if (alive(v) && int(blk[v]) * 4 + J >= limit) {
-                        stop(v);
-                        if constexpr (MODE == 0) {
-                            pend[v] = true;
-                            if (limit < l.max_steps) redo = true;
-                            else atomicOr(l.status, kStatusStepLimit);
-                            if (32 * v + lane == base(v)) steps += (unsigned long long)l.max_steps;
-                        } else {
-                            cut[v] = true;
-                        }
-                    }
-                }
-            }
+        auto step = [&](auto Jc, const float (&z)[V][4]) {
+            constexpr int J = decltype(Jc)::value;
+            const int BO = (j0 + J) * ROWB;
             // publish this step's (d, previous step) of every slot
 #pragma unroll
             for (int v = 0; v < V; ++v)
@@ -663,8 +684,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             }
             if (__any_sync(kAll, bad)) repair(posb + BO, fd, fp);
             // Eq. 1 (a successor at +inf is never within theta: the free branch)
-            float S[V], dn[V];
-            bool fv[V], fin = false;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 float kv, thv, Pv, sgv, muv;
@@ -685,101 +704,91 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 const float Rc = responsiveness<LAW>(kv, d[v], invL, t0r, int(blk[v]) * 4 + j0 + J, invTr);
                 const bool blocked = !(__fsub_rn(fd[v], d[v]) > thv);
                 float Sv = blocked ? __fmul_rn(Rc, fminf(pv[v], fp[v]))
-                                   : __fmul_rn(__fmul_rn(Rc, Pv), __fmaf_rn(sgv, J == 0 ? z[v][0] : J == 1 ? z[v][1] : J == 2 ? z[v][2] : z[v][3], muv));
+                                   : __fmul_rn(__fmul_rn(Rc, Pv), __fmaf_rn(sgv, z[v][J], muv));
                 Sv = fmaxf(Sv, kStepFloor);
-                S[v] = Sv;
-                dn[v] = __fadd_rn(d[v], Sv);
-                fv[v] = dn[v] >= L && (MODE == 0 || d[v] < L);
-                fin |= fv[v];
-            }
-            if constexpr (MODE == 1) {
-                // place mode: a crossing is recorded with its key (sub-step, within-step crossing
-                // time tau, slot) and placed at the block's end; tau > 0, so its bit pattern orders
-                // like its value, and key order is the order of finish with ties to the lower
-                // competitor index (the slot order within a segment)
-                if (__any_sync(kAll, fin)) {
-                    blk_fin = true;
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        if (fv[v]) {
-                            // tau joins the key at the block's end (one division there, none here)
-                            st.fsub[32 * v + lane] = uint8_t(j0 + J);
-                            st.fcross[32 * v + lane] = make_float2(d[v], S[v]);
-                        }
-                    }
-                }
-            } else if (__any_sync(kAll, fin)) {
-                // win mode: least (tau, slot) per segment, at once; tau > 0, so its bit pattern
-                // orders like its value
-                blk_fin = true;
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    if (fv[v]) {
-                        const float tau = __fdiv_rn(__fsub_rn(L, d[v]), S[v]);
-                        atomicMin(&st.key[base(v)], (static_cast<unsigned long long>(__float_as_uint(tau)) << 32) |
-                                                      unsigned(32 * v + lane));
-                    }
-                }
-                __syncwarp();
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    if (alive(v)) {
-                        const int sb = base(v);
-                        const unsigned long long kw = st.key[sb];
-                        if (kw != kNoKey) {
-                            const int slot = 32 * v + lane;
-                            if (int(unsigned(kw)) == slot) atomicAdd(&st.wins[BBE_INDEX(slot - sb, 32, l.status)], 1);
-                            dn[v] = kDead;
-                            fo[v] = kSent;
-                            pend[v] = true;
-                            if (slot == sb) steps += (unsigned long long)(blk[v] * 4u + unsigned(j0 + J) + 1u);
-                        }
-                    }
-                }
-                __syncwarp();
-#pragma unroll
-                for (int v = 0; v < V; ++v)
-                    if (fv[v]) st.key[base(v)] = kNoKey;
-            }
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                d[v] = dn[v];
-                pv[v] = S[v];
+                d[v] = __fadd_rn(d[v], Sv);
+                pv[v] = Sv;
             }
         };
 
-        // blocks before one in which a rollout could reach max_steps (the check starts there)
-        unsigned left = limit >= 4 ? unsigned(limit - 4) / 4u + 1u : 0u;
-        // warp-uniform: the last block may have changed which slots run (a finish, a cut-off);
-        // after a block without either the reduction below would find nothing to do
-        bool blk_event = true;
-        for (;;) {
-            if (blk_event) {
-            blk_event = false;
-            // segments that finished in the last block start their next rollout; one reduction
-            // says whether any did and whether anything still runs
-            bool pany = false, aany = false;
+        // blocks before one at whose end a rollout can have run `limit` steps: no slot is further into
+        // its rollout than the blocks the work item has run, so a warp-uniform count-down rules the
+        // check out in all but the longest items
+        unsigned left = unsigned(max(limit, 1) - 1) / 4u;
+        for (bool live = k_count > 0u; live;) {
+            // the block's normals: one Philox4x32-10 output per slot, counter (k, t >> 2, c, race)
+            float z[V][4];
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                draw_block<DIST>(st.ph[32 * v + lane], PS ? st.pha[kra[v] - st.kr] : pha[v], blk[v], l.round_key, z[v]);
+            if constexpr (MODE == 0) {
+                // two copies of the step, run twice (the second time with the block's other two
+                // normals): with four, the steps and their repairs overflow the instruction cache where
+                // overtakes are frequent (700 bunched races of 13: 15.3 instead of 14.6 ms; spread races
+                // without overtakes lose 1 to 2 %)
+#pragma unroll 1
+                for (;;) {
+                    step(std::integral_constant<int, 0>{}, z);
+                    step(std::integral_constant<int, 1>{}, z);
+                    if (j0 != 0) break;
+                    j0 = 2;
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        z[v][0] = z[v][2];
+                        z[v][1] = z[v][3];
+                    }
+                }
+                j0 = 0;
+            } else {
+                step(std::integral_constant<int, 0>{}, z);
+                step(std::integral_constant<int, 1>{}, z);
+                step(std::integral_constant<int, 2>{}, z);
+                step(std::integral_constant<int, 3>{}, z);
+            }
+            const bool chk = left == 0u;
+            if (!chk) --left;
+            bool event = false;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                pany |= pend[v];
-                aany |= alive(v);
+                ++blk[v];
+                event |= d[v] >= L && (MODE == 0 || st.pos[0][32 * v + lane].x < L);
             }
-            const unsigned state = __reduce_or_sync(kAll, (pany ? 1u : 0u) | (aany ? 2u : 0u));
-            if (state & 1u) {
-                if constexpr (MODE == 1) tally_completed();
+            if (chk) {
 #pragma unroll
-                for (int v = 0; v < V; ++v)
-                    if (pend[v] && 32 * v + lane == base(v)) {
-                        st.segk[32 * v + lane] = atomicAdd(&st.next_k, 1u);
-                        if constexpr (MODE == 1) pl_n[32 * v + lane] = 0;
-                    }
+                for (int v = 0; v < V; ++v) event |= alive(v) && int(blk[v]) * 4 >= limit;
+            }
+            if (!__any_sync(kAll, event)) continue;
+
+            // rollouts have ended: the segments that ran them take the next ones
+            if constexpr (MODE == 0) {
+                win_end(chk);
+                if (chk && __any_sync(kAll, redo)) break;
+            } else {
+                place_end(chk);
                 __syncwarp();
+                tally_completed();
+            }
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    if (!pend[v]) continue;
+            for (int v = 0; v < V; ++v) {
+                const int slot = 32 * v + lane;
+                const bool lead = pend[v] && slot == base(v);
+                const unsigned m = __ballot_sync(kAll, lead);
+                if (lead) {
+                    st.segk[slot] = next_k + unsigned(__popc(m & ((1u << lane) - 1u)));
+                    if constexpr (MODE == 1) pl_n[slot] = 0;
+                }
+                next_k += unsigned(__popc(m));
+            }
+            __syncwarp();
+            live = false;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                if (pend[v]) {
                     pend[v] = false;
                     const int slot = 32 * v + lane, sb = base(v);
                     const unsigned knew = st.segk[sb];
+                    d[v] = kDead;
+                    fo[v] = kSent;
                     if (knew < kend) {
                         const int c = slot - sb;
                         set_stream(slot, knew, c);
@@ -787,76 +796,16 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                         d[v] = st.d0[c];
                         pv[v] = st.prev0[c];
                         const int r0 = st.rank0[c];
-                        fo[v] = r0 + 1 < n ? (sb + st.byrank0[r0 + 1]) * int(sizeof(float2)) : kSent;
-                        const int a = st.rbase[slot] + r0;
+                        if (r0 + 1 < n) fo[v] = (sb + st.byrank0[r0 + 1]) * int(sizeof(float2));
+                        const int a = 1 + 2 * sb + r0;
                         st.order[a] = uint8_t(slot);
                         st.at[slot] = uint8_t(a);
                     }
                 }
-                __syncwarp();
-                bool any_alive = false;
-#pragma unroll
-                for (int v = 0; v < V; ++v) any_alive |= alive(v);
-                if (!__any_sync(kAll, any_alive)) break;
-            } else if (!(state & 2u)) {
-                break;
+                live |= alive(v);
             }
-            }
-
-            // the block's normals: one Philox4x32-10 output per slot, counter (k, t >> 2, c, race)
-            float z[V][4];
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                draw_block<DIST>(st.ph[32 * v + lane], st.pha[32 * v + lane], blk[v], l.round_key, z[v]);
-            // no slot is further into its rollout than the blocks the work item has run, so a
-            // warp-uniform count-down rules out the step limit in all but the longest items
-            bool near_limit = false;
-            if (left == 0u) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) near_limit |= alive(v) && int(blk[v]) * 4 + 4 > limit;
-            } else {
-                --left;
-            }
-            blk_fin = false;
-            if (left == 0u && __any_sync(kAll, near_limit)) {
-                blk_event = true;
-#pragma unroll 1
-                for (int J = 0; J < 4; ++J) step(J, std::true_type{}, z);
-                if constexpr (MODE == 1) block_end();
-                else if (__any_sync(kAll, redo)) break;
-            } else {
-                if constexpr (MODE == 0) {
-                    // two copies of the step, run twice (the second time with the block's other two
-                    // normals): with four, the step, its repair and its finish overflow the
-                    // instruction cache where overtakes are frequent (700 bunched races of 13: 19.4
-                    // instead of 15.8 ms; spread races without overtakes lose 2 %)
-                    j0 = 0;
-#pragma unroll 1
-                    for (;;) {
-                        step(std::integral_constant<int, 0>{}, std::false_type{}, z);
-                        step(std::integral_constant<int, 1>{}, std::false_type{}, z);
-                        if (j0 != 0) break;
-                        j0 = 2;
-#pragma unroll
-                        for (int v = 0; v < V; ++v) {
-                            z[v][0] = z[v][2];
-                            z[v][1] = z[v][3];
-                        }
-                    }
-                    j0 = 0;
-                } else {
-                    step(std::integral_constant<int, 0>{}, std::false_type{}, z);
-                    step(std::integral_constant<int, 1>{}, std::false_type{}, z);
-                    step(std::integral_constant<int, 2>{}, std::false_type{}, z);
-                    step(std::integral_constant<int, 3>{}, std::false_type{}, z);
-                }
-                if constexpr (MODE == 1) {
-                    if (blk_fin) block_end();
-                }
-                blk_event = blk_event || blk_fin;
-            }
-#pragma unroll
-            for (int v = 0; v < V; ++v) ++blk[v];
+            live = __any_sync(kAll, live);
+            __syncwarp();
         }
 
         if (MODE == 0 && __any_sync(kAll, redo)) continue;
@@ -879,16 +828,17 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
 }
 
 // Dynamic shared memory of a block: the warps' stages, then in place mode each warp's place
-// lists (3 x 32 V bytes) and [competitor][place] table (place_cells ints).
+// lists (2 x 32 V bytes) and [competitor][place] table (place_cells ints).
 template <int V, int MODE>
 size_t win_stage_bytes(int block, int place_cells)
 {
     const size_t warps = size_t(block / 32);
-    return warps * sizeof(WinStage<V>) + (MODE == 1 ? warps * (3 * 8 * V + size_t(place_cells)) * sizeof(int) : 0);
+    return warps * sizeof(WinStage<V, MODE>) + (MODE == 1 ? warps * (16 * V + size_t(place_cells)) * sizeof(int) : 0);
 }
 
 // The largest place table a launch may ask for (32 competitors x 32 places).
 constexpr int kMaxPlaceCells = 32 * 32;
+static_assert(16 * (sizeof(WinStage<4, 1>) + 4 * (16 * 4 + kMaxPlaceCells)) <= 227 * 1024, "the largest block");
 
 template <int V, int LAW, int MODE>
 cudaError_t launch_win_vl(const RolloutLaunch &l, cudaStream_t stream)
