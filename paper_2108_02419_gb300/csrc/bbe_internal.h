@@ -63,7 +63,7 @@ struct RolloutLaunch {
     int32_t *next;            // [n_races] tickets' worth of rollouts taken, zeroed before each launch; null: none
     int32_t per_lane;         // with next: rollouts per segment that a warp takes at a time, ..
     int32_t most;             // .. and in all, unless one ticket is worth more
-    int32_t contenders;       // win counts: advance only the competitors that can matter (contender_line)
+    int32_t contenders;       // advance only the competitors that can matter (contender_mask)
     int32_t *counts;          // [n_total]
     unsigned long long *steps;  // [n_races] or null
     int32_t *status;          // device status bits

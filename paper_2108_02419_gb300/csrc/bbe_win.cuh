@@ -24,8 +24,8 @@
 // A finished segment takes its next rollout index from a per-warp counter, so the segments of
 // a work item stay busy until its rollouts run out.
 //
-// Who is advanced.  For win counts only the competitors that can matter to the first finish are
-// (contender_line); they take the slots, so a warp has room for more segments.  A work item is a
+// Who is advanced.  Only the competitors that can matter to the first finish, or the first K, are
+// (contender_mask); they take the slots, so a warp has room for more segments.  A work item is a
 // ticket for some of a race's rollouts, and the warp takes as many as its segments can share.
 //
 // Finishing.  A rollout that ends waits for the block's end in any case, and what its slots do until
@@ -59,6 +59,7 @@ namespace win {
 
 constexpr unsigned kAll = 0xffffffffu;
 constexpr unsigned long long kNoKey = ~0ull;
+constexpr unsigned kRedo = 64;
 constexpr int kPlaced = 128;           // place mode: a segment's K places are filled, at this step of the block
 constexpr unsigned kNone = ~0u;       // win mode: a segment without a finish, ..
 constexpr unsigned kCut = kNone - 1u;  // .. and one whose rollout has run its last step without one
@@ -73,7 +74,11 @@ struct WinStage {
     unsigned pha[32];                   // per competitor: StreamWords::a, the same for all rollouts
     float d0[32], prev0[32];            // per competitor: start state of every rollout
     uint4 ph[NS];                       // per slot: the current rollout's Philox constants (StreamWords)
-    unsigned segk[NS];                  // by segment base: rollout index handed to a restart
+    unsigned segk[NS];                  // by segment base: its rollout
+    // rollouts to run again with everybody: a warp takes no more new ones once kRedo are listed
+    static constexpr bool kContenders = MODE == 0 || V <= 2;
+    unsigned redo[kContenders ? kRedo + NS : 1];
+    unsigned n_redo, rest[2];           // how many; first and end of those not begun for their number
     int wins[MODE == 0 ? 32 : 1];       // wins per competitor in the current work item
     // by segment base; win mode: the block's least (step, tau) and the first slot that has it; place
     // mode: the least crossing key not yet placed
@@ -106,85 +111,108 @@ __device__ __forceinline__ float warp_max(float v)
     return v;
 }
 
-// The contenders of a race.  A first finisher is decided among the competitors near the front, and
-// Eq. 1 passes influence from front to back only, so a competitor that is certain to stay short of
-// the line until a rollout ends cannot change who wins it, nor when.  contender_line returns a
-// position such that, in every rollout that ends within H steps (H is set here), the competitors
-// behind it have no effect on the first finisher: a rollout of the others alone, each on its own
-// stream, has the same winner and the same number of steps.  -inf: nobody is ruled out.
+// The contenders of a race.  The first K finishers are decided among the competitors near the front, and
+// Eq. 1 passes influence from front to back only, so a competitor that is certain to stay short of the
+// line until a rollout ends cannot change its first K places, nor when they are filled.
+// contender_mask returns the competitors that are not ruled out so: in every rollout that ends within
+// H steps (H is set here), a rollout of these alone, each on its own stream, has the same first K
+// finishers and the same number of steps.
 //
-// The bound, for any draws.  A free step is at most F = max R P (mu + z_max sigma) (the generator's
-// |z| is bounded: u1 >= 2^-24 gives a radius of at most 5.7681; sqrt(3) and 1 for the other two
-// distributions) and at least the previous steps given.  A blocked step is R min(own previous step, that
-// of the competitor in front), so it exceeds F only for a competitor whose R can exceed 1 (the set
-// D; lambda is the largest R), and then
-//   S_c(t) > lambda^k F  =>  S(t-1) > lambda^(k-1) F for c and for the one in front of it, within theta.
-// Of the competitors in a stretch of track with S(t) > lambda^k F the foremost has one in front that is
-// not among them, so each level down has one member more: S_c(t) > lambda^k F takes k + 1 members of D
-// close together, whose start positions span at most G(t) + k theta, where G(t) bounds what anyone
-// covers in t steps.  With w_k the least span of k + 1 members of D at the start,
-//   G(t+1) = G(t) + F lambda^#{k : w_k <= G(t) + n theta}
-// bounds everyone's advance.  A competitor starting behind L - G(H) is short of the line for H steps; so
-// is one that gets affected by it (it was passed, so it was behind it at that time, and G(t) bounds it
-// from there on); so whoever crosses first within H steps was never behind any of them.  Rounding is
-// covered by the factors and the margin below.
+// The bound, for any draws.  E_i(t) bounds the position after t steps of every competitor that starts at or
+// behind rank i (ranks by start position) and of everyone that one of them has affected (the affected
+// were behind it, so the bound holds for them from there on).  A free step is at most F = max R P (mu +
+// z_max sigma), the largest over the competitors (the generator's |z| is bounded: u1 >= 2^-24 gives a
+// radius of at most 5.7681; sqrt(3) and 1 for the other two distributions) and at least the previous
+// steps given.  A blocked step is R min(own previous step, that of the competitor in front), so with lambda
+// the largest R where it happens,
+//   S_c(t) > lambda^k F  =>  S(t-1) > lambda^(k-1) F for c and for the one in front of it, within theta,
+// and the foremost of those who have S(t-i) > lambda^(k-i) F has one in front that is not among them:
+// k levels take k members whose R can exceed 1, each within n theta of another at some of the last k
+// steps.  A member that was there i steps ago has fallen back since by at most i steps' difference
+// between the largest step and F, by less than M in all.  So if j is the rearmost member, c is at most M
+// ahead of E_j, the others rank above j and started behind E_j + M + n theta, and those are counted
+// (k_j, lambda_j):
+//   V_j = F lambda_j^k_j,   E_i(t+1) = max over j <= i of min(E_j(t) + M, E_i(t)) + V_j.
+// M for step t follows from the levels of the step before, which a step exceeds by one at most.  Rounding is
+// covered by the factors and the margins.  A competitor is ruled out when its E stays short of the
+// line for H steps.  (With one bound for everybody's advance, the closest groups anywhere on the
+// track count against all: 10 contenders of 20 at the mean in the uniform batch, 4.8 with this one.)
 //
-// H is an estimate of the first finish with a margin of five standard deviations; a rollout that
-// is still running after H steps makes the warp redo its work item with a longer H, then with everybody.
-// x: n floats of scratch.  Called by the whole warp; lane c < n holds competitor c.
+// H is an estimate of the K-th finish with a margin of three standard deviations; the few rollouts
+// that are still running after H steps are run again with everybody.
+// x: 3 n floats of scratch.  Called by the whole warp; lane c < n holds competitor c.
 template <int DIST, int LAW>
-__device__ __forceinline__ float contender_line(float *x, int n, int lane, float d, float mu, float sigma, float P,
-                                                float kr, float prev, float theta, float L, float t0, float invT,
-                                                float stretch, int &H)
+__device__ __forceinline__ unsigned contender_mask(float *x, int n, int lane, float d, float mu, float sigma, float P,
+                                                   float kr, float prev, float theta, float L, float invL, float t0,
+                                                   float invT, int K, int &H)
 {
     const bool on = lane < n;
+    const unsigned everybody = kAll >> (32 - n);
     constexpr float zmax = DIST == BBE_DIST_NORMAL ? 5.769f : (DIST == BBE_DIST_UNIFORM ? 1.7321f : 1.0f);
-    // expected finish at the R of the middle of the way, and the horizon
+    // expected finish at the R of the middle of the way, and the horizon: the K-th least with its margin
     float T = (L - d) / (mu * P);
-    T /= 1.0f + (LAW == BBE_LAW_TIME ? kr * (fminf((t0 + 0.5f * T) * invT, 1.0f) - 0.5f) : 0.5f * kr * d / L);
-    const float h = warp_min(on ? stretch * (1.03f * T + 5.0f * sigma * sqrtf(T) / mu + 3.0f) : INFINITY);
-    if (!(h < 1e6f)) return -INFINITY;
-    H = int(h) + 1;
-    // the largest R of each competitor (linear in the position or the time: at an end of its range)
-    float R;
-    if (LAW == BBE_LAW_TIME) {
-        const float u0 = fminf(t0 * invT, 1.0f), u1 = fminf((t0 + float(H)) * invT, 1.0f);
-        R = 1.0f + fmaxf(kr * (u0 - 0.5f), kr * (u1 - 0.5f));
-    } else {
-        R = 1.0f + fmaxf(kr * (d / L - 0.5f), 0.5f * kr);
-    }
-    R *= 1.00001f;
-    const float F = 1.0001f * fmaxf(warp_max(on ? fmaxf(prev, R * P * (mu + zmax * sigma)) : 0.0f), kStepFloor);
-    const float dmin = warp_min(on ? d : INFINITY);
-    if (!(L - float(H) * F > dmin)) return -INFINITY;  // not even at the free pace
-    const float lambda = fmaxf(warp_max(on ? R : 0.0f), 1.0f);
-    const float margin = 1e-4f * L + float(n) * warp_max(on ? theta : 0.0f);
-    const bool grows = on && R > 0.9999f;
-    const unsigned D = __ballot_sync(kAll, grows);
-    const int m = __popc(D);
-    int rank = 0;
+    T /= 1.0f + (LAW == BBE_LAW_TIME ? kr * (fminf((t0 + 0.5f * T) * invT, 1.0f) - 0.5f) : 0.5f * kr * d * invL);
+    const float h = on ? T + 3.0f * sigma * sqrtf(T) / mu + 1.0f : INFINITY;
+    int rank = 0, hrank = 0;  // by (start position, index) and by (horizon, index)
     for (int i = 0; i < n; ++i) {
-        const float di = __shfl_sync(kAll, d, i);
-        rank += ((D >> i) & 1u) && (di < d || (di == d && i < lane)) ? 1 : 0;
+        const float di = __shfl_sync(kAll, d, i), hi = __shfl_sync(kAll, h, i);
+        rank += di < d || (di == d && i < lane) ? 1 : 0;
+        hrank += hi < h || (hi == h && i < lane) ? 1 : 0;
     }
-    if (grows) x[rank] = d;
+    const float hk = warp_max(on && hrank < K ? h : 0.0f);
+    const float margin = float(n) * warp_max(on ? theta : 0.0f);
+    if (!(hk < 1e6f) || !(margin < L)) return everybody;
+    H = int(hk) + 1;
+    // R is linear in the position or the time: largest at an end of its range
+    const float lo = LAW == BBE_LAW_TIME ? fminf(t0 * invT, 1.0f) : d * invL;
+    const float end = LAW == BBE_LAW_TIME ? fminf((t0 + float(H)) * invT, 1.0f) : (L + margin) * invL;
+    const float Rlo = 1.0f + kr * (lo - 0.5f);
+    const float R = 1.00001f * fmaxf(Rlo, 1.0f + kr * (end - 0.5f));
+    const float F = 1.0001f * fmaxf(warp_max(on ? fmaxf(prev, R * P * (mu + zmax * sigma)) : 0.0f), kStepFloor);
+    const float dmin = warp_min(on ? d : INFINITY), goal = 0.9999f * L;
+    if (!(goal - float(H) * F > dmin)) return everybody;  // not even at the free pace
+    const float lambda = 1.00001f * fmaxf(warp_max(on ? R : 0.0f), 1.0f);  // anywhere
+    // from here on lane i holds rank i
+    if (on) {
+        x[rank] = d;
+        x[n + rank] = kr;
+        x[2 * n + rank] = Rlo;
+    }
     __syncwarp();
-    float w = INFINITY;  // least span of lane + 1 members of D
-    for (int i = 0; i + lane < m; ++i) w = fminf(w, x[i + lane] - x[i]);
-    __syncwarp();
-    float G = 0.0f;
+    float E = on ? x[lane] : INFINITY, M = margin;
+    float rise = 0.0f, Rmax = 1.0f;  // of the ranks lane .. next - 1: the largest kr, and R at the range's start
+    int next = lane, early = 0, late = 0;  // those whose R exceeds 1 there, and those later on only
     for (int t = 0; t < H;) {
-        const int k = __popc(__ballot_sync(kAll, w <= G + margin));
-        const float V = 1.0001f * F * powf(lambda, float(k));
-        const float next = __shfl_sync(kAll, w, k & 31);
-        int steps = H - t;
-        if (k < m) steps = min(steps, int(fminf((next - margin - G) / V, 1e6f)) + 1);
-        steps = max(steps, 1);
-        G += float(steps) * V;
-        t += steps;
-        if (!(L - G > dmin)) return -INFINITY;
+        while (next < n && x[next] <= E + M + margin) {
+            const float k1 = x[n + next], r1 = x[2 * n + next];
+            Rmax = fmaxf(Rmax, r1);
+            if (r1 > 0.9999f) ++early;
+            else if (k1 > 0.0f) ++late;
+            rise = fmaxf(rise, k1);
+            ++next;
+        }
+        const float now = LAW == BBE_LAW_TIME ? fminf((t0 + float(t)) * invT, 1.0f) : fminf((E + M + margin) * invL, end);
+        const int k = early + (now > 0.4999f ? late : 0);
+        const float lam = 1.00001f * fmaxf(Rmax, 1.0f + rise * (now - 0.5f));
+        const float V = on ? 1.0001f * F * powf(lam, float(k)) : 0.0f;
+        float En = E + V;
+        for (int j = 0; j + 1 < n; ++j) {
+            const float Ej = __shfl_sync(kAll, E, j), Vj = __shfl_sync(kAll, V, j);
+            if (j < lane) En = fmaxf(En, fminf(Ej + M, E) + Vj);
+        }
+        E = En;
+        if (__shfl_sync(kAll, E, 0) >= goal) {
+            __syncwarp();
+            return everybody;
+        }
+        const int km = __reduce_max_sync(kAll, on ? k : 0);
+        M = fmaxf(M, margin + float(km) * F * (1.0002f * powf(lambda, float(km)) - 1.0f));
+        ++t;
     }
-    return L - 1.001f * G - margin;
+    const float bound = __shfl_sync(kAll, E, rank & 31);
+    const bool out = on && !(bound >= goal);
+    __syncwarp();
+    return everybody & ~__ballot_sync(kAll, out);
 }
 
 template <int DIST>
@@ -207,13 +235,14 @@ __device__ __forceinline__ void draw_block(const uint4 &q, uint32_t a, uint32_t 
     }
 }
 
-// Registers per thread.  Win counts: 80 for two slots per lane (6 resident 4-warp blocks per SM) and
-// 64 for one; with 72 and 56 (7 and 9 blocks) a pass over 4096 races of 20 takes 57.1 instead of
-// 54.7 ms and one small race, run in that layout, 42 instead of 37 us.  Place mode spills nothing at 72, and fewer warps
-// cost it 1 %.  Three and four slots per lane read their parameters from shared memory.
+// Registers per thread: 80 for two to four slots per lane (6 resident 4-warp blocks per SM); with 72
+// (7 blocks) places to the third of 512 races of 20 take 16.3 instead of 15.2 ms, win counts the same
+// (4096 races: 31.7 and 32.2).  64 for one slot per lane, the layout of the smallest calls, which gain
+// from fewer spills, not from more warps (one small race 37 us, 42 at 56).  Three and four slots per
+// lane read their parameters from shared memory.
 template <int V, int MODE>
 struct WinRegs {
-    static constexpr int value = V == 1 ? (MODE == 0 ? 64 : 48) : (V == 2 ? (MODE == 0 ? 80 : 72) : 80);
+    static constexpr int value = V == 1 ? (MODE == 0 ? 64 : 56) : 80;
 };
 // Parameters read from shared memory each step instead of held in registers.
 template <int V>
@@ -275,10 +304,16 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             if (int64_t(taken) * w.k_count >= Rr) continue;
         }
         unsigned k_begin = unsigned(w.k_begin), k_count = unsigned(w.k_count);
-        // win counts: first with the contenders alone, and again only if a rollout ran past
-        // the horizon that they were chosen for
-        for (int attempt = 0;; ++attempt) {
+        const int K = MODE == 1 ? min(l.places, n_race) : 1;  // places run per rollout
+        // First with the contenders alone; then, with everybody, the rollouts that ran past the horizon
+        // that those were chosen for, and what was not begun for the number of those.
+        enum { kFirst, kListed, kRest };
+        for (int pass = kFirst;;) {
         __syncwarp();
+        if (lane == 0) {
+            st.n_redo = 0u;
+            if (pass == kFirst) st.rest[0] = st.rest[1] = 0u;
+        }
         // stage the race: lane j < n_race loads competitor j (coalesced)
         float my_d0 = INFINITY, my_mu = 1.0f, my_sg = 0.0f, my_P = 1.0f, my_th = 0.0f, my_kr = 0.0f, my_pv = 0.0f;
         if (lane < n_race) {
@@ -295,25 +330,21 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         // that makes room for more segments
         unsigned keep = kAll >> (32 - n_race);
         int limit = l.max_steps;  // a rollout that reaches it ends undecided
-        if constexpr (MODE == 0) {
-            if (l.contenders && attempt < 2 && n_race > 1) {
-                int H = 0;
-                const float line = contender_line<DIST, LAW>(reinterpret_cast<float *>(posb), n_race, lane, my_d0, my_mu, my_sg,
-                                                            my_P, my_kr, my_pv, my_th, L, t0r, invTr,
-                                                            attempt == 0 ? 1.0f : 1.4f, H);
-                const unsigned front = __ballot_sync(kAll, lane < n_race && my_d0 >= line);
-                const int nf = __popc(front);
-                if (nf > 0 && (l.seg_cap > 0 ? min(NS / nf, l.seg_cap) > min(NS / n_race, l.seg_cap) : NS / nf > NS / n_race)) {
-                    keep = front;
-                    limit = min(limit, H);
-                }
+        if (Stage::kContenders && pass == kFirst && l.contenders && K < n_race) {
+            int H = 0;
+            const unsigned front = contender_mask<DIST, LAW>(reinterpret_cast<float *>(st.ph), n_race, lane, my_d0, my_mu,
+                                                             my_sg, my_P, my_kr, my_pv, my_th, L, invL, t0r, invTr, K, H);
+            const int nf = __popc(front);
+            if (nf >= K && (l.seg_cap > 0 ? min(NS / nf, l.seg_cap) > min(NS / n_race, l.seg_cap) : NS / nf > NS / n_race)) {
+                keep = front;
+                limit = min(limit, H);
             }
         }
         const int n = __popc(keep);
         const int nseg = l.seg_cap > 0 ? min(NS / n, l.seg_cap) : NS / n;  // segments of this warp
-        if (l.next != nullptr && attempt == 0) {
+        if (l.next != nullptr && pass == kFirst) {
             // as many rollouts as give every segment its share, in multiples of the ticket's
-            const int mult = MODE == 0 ? max(1, min(l.per_lane * nseg, l.most) / w.k_count) : 1;
+            const int mult = max(1, min(l.per_lane * nseg, l.most) / w.k_count);
             int first = 0;
             if (lane == 0) first = atomicAdd(l.next + r, mult);
             const int64_t k = int64_t(__shfl_sync(kAll, first, 0)) * w.k_count;
@@ -322,7 +353,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             const int64_t share = int64_t(mult) * w.k_count;
             k_count = unsigned(share < Rr - k ? share : Rr - k);
         }
-        bool redo = false;  // a rollout of the contenders ran past their horizon
         const bool kept = (keep >> lane) & 1u;
         int rank = 0;  // by (d0, index)
         for (int i = 0; i < n_race; ++i) {
@@ -356,15 +386,14 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             st.order[2 * NS + lane] = uint8_t(NS);
             st.flag[2 * NS + lane] = 0;
         }
-        const int K = MODE == 1 ? min(l.places, n) : 1;  // places run per rollout
         if constexpr (MODE == 1) {
             for (int i = lane; i < n * K; i += 32) pl_cnt[i] = 0;
         }
         __syncwarp();
 
         // unsigned: rollout indices stay below 2^31 + 2^7
-        const unsigned kend = k_begin + k_count;
-        unsigned next_k = k_begin + unsigned(nseg);  // warp-uniform: the next segment that is free takes it
+        unsigned kend = k_begin + k_count;
+        unsigned next_k = k_begin + unsigned(nseg);  // warp-uniform (as kend): the next segment that is free takes it
 
         // per slot: segment base, competitor parameters, state, front address, rollout, block
         int fo[V];
@@ -374,11 +403,11 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         const float *kra[V];   // register-lean variant: this slot's kappa (2 rho - 1)
         // a slot that runs no rollout has no position (NaN): it is never out of order, never over
         // the line, and stays so without a test in the step
-        bool pend[V];  // rollout ended, to restart
         auto alive = [&](int v) { return d[v] == d[v]; };
         auto base = [&](int v) { return int(st.base[32 * v + lane]); };
         // slot's stream for rollout k (competitor c of the advanced ones)
         auto set_stream = [&](int slot, unsigned k, int c) {
+            if (pass == kListed && k < kend) k = st.redo[BBE_INDEX(k, kRedo + NS, l.status)];
             const StreamWords q = stream_words(k, uint32_t(st.comp[c]), rid, l.round_key);
             st.ph[slot] = make_uint4(q.d, q.e, q.f, q.g);
         };
@@ -393,11 +422,11 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             const int c = used ? slot - seg * n : 0;
             const unsigned k = k_begin + unsigned(seg);
             const bool run = used && k < kend;
+            if (slot == sb) st.segk[slot] = k;
             st.base[slot] = uint8_t(sb);
             const int rb = 1 + 2 * sb;
             st.at[slot] = uint8_t(rb);
             set_stream(slot, k, c);
-            pend[v] = false;
             blk[v] = 0;
             if constexpr (PS) {
                 pqa[v] = &st.pq[c];
@@ -521,7 +550,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         // Win mode, the end of a block with a crossing (or, chk, one in which a rollout may have run its
         // last step): the least key (step, tau) of each segment, then the least slot that has it.  tau =
         // (L - d) / S is in [0, 2], so its bit pattern less one orders like its value and fits in 30 bits.
-        auto win_end = [&](bool chk) {
+        auto win_end = [&](bool chk, bool (&pend)[V], bool (&again)[V]) {
             unsigned mine[V], kw[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -550,9 +579,12 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 const int slot = 32 * v + lane;
                 if (!pend[v] || slot != base(v)) continue;
                 if (kw[v] == kCut) {
-                    if (limit < l.max_steps) redo = true;
-                    else atomicOr(l.status, kStatusStepLimit);
-                    steps += (unsigned long long)l.max_steps;
+                    if (limit >= l.max_steps) {
+                        atomicOr(l.status, kStatusStepLimit);
+                        steps += (unsigned long long)l.max_steps;
+                    } else {
+                        again[v] = true;
+                    }
                 } else {
                     atomicAdd(&st.wins[BBE_INDEX(int(st.key.win[1][slot]) - slot, 32, l.status)], 1);
                     steps += (unsigned long long)(blk[v] * 4u - 3u + (kw[v] >> 30));
@@ -564,7 +596,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         // Place mode, the same: the block's crossings of each segment take the next places one at a
         // time in key order (step, tau, slot), and a segment whose K-th place is filled ends its
         // rollout; one stopped at max_steps that did not end earlier counts for nobody.
-        auto place_end = [&](bool chk) {
+        auto place_end = [&](bool chk, bool (&pend)[V], bool (&again)[V]) {
             unsigned long long fk[V];
             int sb[V];
             bool more = false;
@@ -619,8 +651,12 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     if (slot == sb[v]) steps += (unsigned long long)(blk[v] * 4u - 3u + filled - kPlaced);
                     pend[v] = true;
                 } else if (chk && int(blk[v]) * 4 >= limit) {
-                    if (slot == sb[v]) steps += (unsigned long long)l.max_steps;
-                    atomicOr(l.status, kStatusStepLimit);
+                    if (limit >= l.max_steps) {
+                        if (slot == sb[v]) steps += (unsigned long long)l.max_steps;
+                        atomicOr(l.status, kStatusStepLimit);
+                    } else {
+                        again[v] = slot == sb[v];
+                    }
                     pend[v] = true;
                 }
             }
@@ -631,7 +667,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         // place and, for the ordered tallies, their order: as one base-n number (the dense
         // tables, K <= 3) and as the order key, the mixed-radix number whose digit j (radix
         // n - j) is the place-j finisher's index among the competitors not yet placed.
-        auto tally_completed = [&]() {
+        auto tally_completed = [&](const bool (&pend)[V]) {
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 const int sb = base(v);
@@ -642,15 +678,15 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     unsigned code = 0u, taken = 0u;
                     unsigned long long key = 0ull;
                     for (int j = 0; j < K; ++j) {
-                        const int cj = pl_ord[sb + j];
-                        code = code * unsigned(n) + unsigned(cj);
-                        key = key * unsigned(n - j) + unsigned(__popc(((1u << cj) - 1u) & ~taken));
+                        const int cj = st.comp[pl_ord[sb + j]];
+                        code = code * unsigned(n_race) + unsigned(cj);
+                        key = key * unsigned(n_race - j) + unsigned(__popc(((1u << cj) - 1u) & ~taken));
                         taken |= 1u << cj;
                     }
                     if (l.orders != nullptr) {
 #if defined(BBE_CHECKED) && BBE_CHECKED
                         unsigned cells = 1u;  // n^K entries in the race's dense table
-                        for (int j = 0; j < K; ++j) cells *= unsigned(n);
+                        for (int j = 0; j < K; ++j) cells *= unsigned(n_race);
 #endif
                         atomicAdd(&l.orders[l.order_off[r] + BBE_INDEX(code, cells, l.status)], 1);
                     }
@@ -760,13 +796,35 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             if (!__any_sync(kAll, event)) continue;
 
             // rollouts have ended: the segments that ran them take the next ones
+            bool pend[V], again[V];  // rollout ended; at a segment's base: it is to be run again with everybody
+#pragma unroll
+            for (int v = 0; v < V; ++v) pend[v] = again[v] = false;
             if constexpr (MODE == 0) {
-                win_end(chk);
-                if (chk && __any_sync(kAll, redo)) break;
+                win_end(chk, pend, again);
             } else {
-                place_end(chk);
+                place_end(chk, pend, again);
                 __syncwarp();
-                tally_completed();
+                tally_completed(pend);
+            }
+            if (Stage::kContenders && chk && limit < l.max_steps) {
+                unsigned n_redo = st.n_redo;
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const unsigned m = __ballot_sync(kAll, again[v]);
+                    if (again[v])
+                        st.redo[BBE_INDEX(n_redo + unsigned(__popc(m & ((1u << lane) - 1u))), kRedo + NS, l.status)] =
+                            st.segk[32 * v + lane];
+                    n_redo += unsigned(__popc(m));
+                }
+                __syncwarp();
+                if (lane == 0) st.n_redo = n_redo;
+                if (n_redo >= kRedo && next_k < kend) {
+                    if (lane == 0) {
+                        st.rest[0] = next_k;
+                        st.rest[1] = kend;
+                    }
+                    kend = next_k;
+                }
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -784,7 +842,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 if (pend[v]) {
-                    pend[v] = false;
                     const int slot = 32 * v + lane, sb = base(v);
                     const unsigned knew = st.segk[sb];
                     d[v] = kDead;
@@ -808,21 +865,31 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             __syncwarp();
         }
 
-        if (MODE == 0 && __any_sync(kAll, redo)) continue;
         // one global atomic per competitor with wins (per competitor and place in place mode), one
-        // per work item for the step total
+        // for the step total
         __syncwarp();
         if constexpr (MODE == 1) {
             for (int i = lane; i < n * K && l.counts != nullptr; i += 32) {
                 const int cc = pl_cnt[i];
-                if (cc != 0) atomicAdd(&l.counts[(off + i / K) * l.places + i % K], cc);
+                if (cc != 0) atomicAdd(&l.counts[(off + st.comp[i / K]) * l.places + i % K], cc);
             }
         } else {
             if (lane < n && st.wins[lane] != 0) atomicAdd(&l.counts[off + st.comp[lane]], st.wins[lane]);
         }
         for (int o = 16; o > 0; o >>= 1) steps += __shfl_xor_sync(kAll, steps, o);
         if (lane == 0 && l.steps != nullptr) atomicAdd(l.steps + r, steps);
-        break;
+        __syncwarp();
+        const unsigned listed = st.n_redo;
+        if (listed > 0u) {
+            pass = kListed;
+            k_begin = 0u;
+            k_count = listed;
+        } else {
+            k_begin = st.rest[0];
+            k_count = st.rest[1] - k_begin;
+            if (pass == kRest || k_count == 0u) break;
+            pass = kRest;
+        }
         }
     }
 }

@@ -92,3 +92,45 @@ def test_step_limit_among_contenders():
     want_counts, want_steps, _ = oracle.batch_counts(rb, max_steps=27)
     assert np.array_equal(counts.cpu().numpy(), want_counts)
     assert np.array_equal(steps.cpu().numpy(), want_steps)
+
+
+@pytest.mark.parametrize("places", [2, 4])
+@pytest.mark.parametrize("name", list(CASES))
+def test_contenders_alone_give_the_first_places(name, places):
+    import torch
+
+    from paper_2108_02419_gb300 import bbe
+
+    rb = CASES[name]()
+    with bbe.Batch(rb) as b:
+        counts, steps = b.places(places)
+        b.status()
+        torch.cuda.synchronize()
+    want_counts, want_steps, st = oracle.batch_places(rb, places)
+    assert st == 0
+    assert np.array_equal(counts.cpu().numpy(), want_counts)
+    assert np.array_equal(steps.cpu().numpy(), want_steps)
+
+
+@pytest.mark.parametrize("name", ["twenty", "full warp", "far blocking", "stuck behind the leader", "time law, late"])
+def test_contenders_alone_give_the_orders(name):
+    # the tables are indexed by all the race's competitors, whoever is advanced
+    import torch
+
+    from paper_2108_02419_gb300 import bbe
+
+    rb = CASES[name]()
+    with bbe.Batch(rb) as b:
+        orders = b.orders(2)[0]
+        keys, hcounts, off, _, _ = b.order_histogram(3)
+        b.status()
+        torch.cuda.synchronize()
+        orders, keys, hcounts = orders.cpu().numpy(), keys.cpu().numpy(), hcounts.cpu().numpy()
+    want, want_h = oracle.batch_orders(rb, 2)[0], oracle.batch_order_histograms(rb, 3)[0]
+    assert np.array_equal(orders, np.concatenate([np.ravel(t) for t in want]) if isinstance(want, list) else np.ravel(want))
+    for r in range(rb.n_races):
+        n = int(rb.race_off[r + 1] - rb.race_off[r])
+        k, c = keys[off[r]:off[r + 1]], hcounts[off[r]:off[r + 1]]
+        used = k != np.uint64(2 ** 64 - 1)
+        got = {tuple(int(x) for x in bbe.bbe_order_key_decode(n, 3, int(key))): int(v) for key, v in zip(k[used], c[used])}
+        assert got == dict(want_h[r]), r
