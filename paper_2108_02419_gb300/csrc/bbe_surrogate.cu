@@ -129,116 +129,128 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p)
 
 // ------------------------------------------------------------------ tile bookkeeping
 
-// barrier of the threads that work on one tile: the whole block, or the threads of one
-// forward tile pipeline (named barrier 1 + pipeline)
-struct BlockSync {
-    __device__ void operator()() const { __syncthreads(); }
-};
+// barrier of the threads of one forward tile pipeline (named barrier 1 + pipeline)
 struct GroupSync {
     int id, count;
     __device__ void operator()() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory"); }
 };
 
+// a tile's races: their indices and first rows ([ns] = rows in use)
 struct RowMap {
-    int row_race[TILE];   // race index of each row (-1: padding)
-    int row_comp[TILE];   // competitor index within its race
-    int row_state[TILE];  // race position within the tile
     int state_row0[MAX_STATES + 1];
-    int state_n[MAX_STATES];
     int state_race[MAX_STATES];
 };
 
-// called by the tile's threads (tid 0..127 at least)
-template <typename Sync>
-__device__ void build_rowmap(RowMap &m, const SgArgs &a, const SgTile &t, int tid, Sync sync)
+// Called by the tile's 128 threads; returns the race slot of row `tid` (-1: padding).  The first rows come
+// from a prefix sum over one warp (two races a lane), a row's slot from a bisection of them: a short
+// chain of dependent loads, which is what this kernel's time is (a serial sum by one thread and a loop
+// over each race's rows made it 2 us longer).
+__device__ int build_rowmap(RowMap &m, const SgArgs &a, const SgTile &t, int tid)
 {
-    if (tid < t.ns) {
-        const int r = a.order[t.s0 + tid];
-        m.state_race[tid] = r;
-        m.state_n[tid] = a.b.race_off[r + 1] - a.b.race_off[r];
-    }
-    sync();
-    if (tid == 0) {
-        int row = 0;
-        for (int i = 0; i < t.ns; ++i) {
-            m.state_row0[i] = row;
-            row += m.state_n[i];
+    static_assert(MAX_STATES == 64, "two races a lane");
+    if (tid < 32) {
+        int n[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            n[h] = 0;
+            const int i = 2 * tid + h;
+            if (i < t.ns) {
+                const int r = a.order[t.s0 + i];
+                m.state_race[i] = r;
+                n[h] = a.b.race_off[r + 1] - a.b.race_off[r];
+            }
         }
-        m.state_row0[t.ns] = row;
-    }
-    if (tid < TILE) m.row_race[tid] = -1;
-    sync();
-    if (tid < t.ns) {
-        const int r0 = m.state_row0[tid];
-        for (int c = 0; c < m.state_n[tid]; ++c) {
-            m.row_race[r0 + c] = m.state_race[tid];
-            m.row_comp[r0 + c] = c;
-            m.row_state[r0 + c] = tid;
+        int sum = n[0] + n[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, sum, o);
+            if (tid >= o) sum += v;
         }
+        if (2 * tid <= t.ns) m.state_row0[2 * tid] = sum - n[0] - n[1];
+        if (2 * tid + 1 <= t.ns) m.state_row0[2 * tid + 1] = sum - n[1];
+        if (tid == 31 && t.ns == MAX_STATES) m.state_row0[MAX_STATES] = sum;
     }
-    sync();
+    __syncthreads();
+    if (tid >= m.state_row0[t.ns]) return -1;
+    int lo = 0, hi = t.ns - 1;  // the last race whose first row is at most tid
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (m.state_row0[mid] <= tid) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
 }
 
-// Input features of tile row `tid` (float32; zeros for padding rows and for tid >= 128): the
-// raw quantities [d/L, (L-d)/5000, mu-16, sigma-1, 2 rho-1] and, per race, the expected finish
-// time T = (L-d)/v with v = mu (1 + 0.1 (2 rho - 1) d/L), its spread s = sigma sqrt(T)/v, the
-// lag behind the race's least T and its z-score, the gaps to the nearest competitors strictly
-// ahead and behind, 1/n, and the catch-up shares.  Called by all threads of the tile.
+// Input features of tile row `tid` (float32; zeros for padding rows, st < 0): the raw quantities [d/L,
+// (L-d)/5000, mu-16, sigma-1, 2 rho-1] and, per race, the expected finish time T = (L-d)/v with v = mu (1
+// + 0.1 (2 rho - 1) d/L), its spread s = sigma sqrt(T)/v, the lag behind the race's least T and its
+// z-score, the gaps to the nearest competitors strictly ahead and behind, 1/n, and the catch-up
+// shares.  Called by the tile's 128 threads; st: the row's race slot.
 struct FeatScratch {
-    float T[TILE], sd[TILE], d[TILE], v[TILE], raw[TILE][RAW];
+    float2 Td[TILE];  // (T, d): what the scan of a race's rows compares
+    float sd[TILE], v[TILE];
 };
 
-template <typename Sync>
-__device__ void tile_features(float (&f)[KIN], FeatScratch &fs, const SgArgs &a, const RowMap &m, int tid, Sync sync)
+__device__ void tile_features(float (&f)[KIN], FeatScratch &fs, const SgArgs &a, const RowMap &m, int tid, int st)
 {
-    if (tid < TILE) {
-        const int r = m.row_race[tid];
-        if (r >= 0) {
-            const int i = a.b.race_off[r] + m.row_comp[tid];
-            const float L = a.b.L[r], d = a.b.d0[i], mu = a.b.mu[i], sigma = a.b.sigma[i], rho = a.b.rho[i];
-            const float frac = d / L;
-            const float v = mu * (1.0f + 0.1f * (2.0f * rho - 1.0f) * frac);
-            const float T = (L - d) / v;
-            fs.T[tid] = T;
-            fs.v[tid] = v;
-            fs.sd[tid] = sigma * sqrtf(T) / v;
-            fs.d[tid] = d;
-            fs.raw[tid][0] = frac;
-            fs.raw[tid][1] = (L - d) / L_SCALE;
-            fs.raw[tid][2] = mu - 16.0f;
-            fs.raw[tid][3] = sigma - 1.0f;
-            fs.raw[tid][4] = 2.0f * rho - 1.0f;
-        }
-    }
-    sync();
 #pragma unroll
     for (int k = 0; k < KIN; ++k) f[k] = 0.0f;
-    if (tid < TILE && m.row_race[tid] >= 0) {
-        const int st = m.row_state[tid];
-        const int r0 = m.state_row0[st], r1 = m.state_row0[st + 1];
-        int kmin = r0, ia = -1, ib = -1;
-        const float dc = fs.d[tid];
-        for (int q = r0; q < r1; ++q) {
-            if (fs.T[q] < fs.T[kmin]) kmin = q;
-            if (fs.d[q] > dc && (ia < 0 || fs.d[q] < fs.d[ia])) ia = q;
-            if (fs.d[q] < dc && (ib < 0 || fs.d[q] > fs.d[ib])) ib = q;
-        }
-        const float ga = ia >= 0 ? fs.d[ia] - dc : 100.0f;
-        const float gb = ib >= 0 ? dc - fs.d[ib] : 100.0f;
-        const float lag = fs.T[tid] - fs.T[kmin];
-        const float vc = fs.v[tid];
-#pragma unroll
-        for (int k = 0; k < RAW; ++k) f[k] = fs.raw[tid][k];
-        f[5] = fs.T[tid] / 100.0f;
-        f[6] = fminf(lag, 100.0f) / 10.0f;
-        f[7] = fs.sd[tid];
-        f[8] = fminf(lag / sqrtf(fs.sd[tid] * fs.sd[tid] + fs.sd[kmin] * fs.sd[kmin] + 0.01f), 20.0f) / 5.0f;
-        f[9] = fminf(ga, 100.0f) / 10.0f;
-        f[10] = 1.0f / float(r1 - r0);
-        f[11] = fminf(gb, 100.0f) / 10.0f;
-        f[12] = (ia >= 0 && vc > fs.v[ia]) ? fminf(ga / (vc - fs.v[ia]) / fs.T[tid], 2.0f) / 2.0f : 1.0f;
-        f[13] = (ib >= 0 && fs.v[ib] > vc) ? fminf(gb / (fs.v[ib] - vc) / fs.T[ib], 2.0f) / 2.0f : 1.0f;
+    const int r0 = st >= 0 ? m.state_row0[st] : 0, r1 = st >= 0 ? m.state_row0[st + 1] : 0;
+    float T = 0.0f, dc = 0.0f, vc = 0.0f, sd = 0.0f;
+    if (st >= 0) {
+        const int r = m.state_race[st];
+        const int i = a.b.race_off[r] + (tid - r0);
+        const float L = a.b.L[r], d = a.b.d0[i], mu = a.b.mu[i], sigma = a.b.sigma[i], rho = a.b.rho[i];
+        const float frac = d / L;
+        const float v = mu * (1.0f + 0.1f * (2.0f * rho - 1.0f) * frac);
+        dc = d;
+        vc = v;
+        T = (L - d) / v;
+        sd = sigma * sqrtf(T) / v;
+        fs.Td[tid] = make_float2(T, d);
+        fs.v[tid] = v;
+        fs.sd[tid] = sd;
+        f[0] = frac;
+        f[1] = (L - d) / L_SCALE;
+        f[2] = mu - 16.0f;
+        f[3] = sigma - 1.0f;
+        f[4] = 2.0f * rho - 1.0f;
     }
+    __syncthreads();
+    if (st < 0) return;
+    // the best so far are held in registers, so the loads of the scan do not wait for one another
+    int kmin = r0, ia = -1, ib = -1;
+    float Tmin = INFINITY, da = 0.0f, db = 0.0f;
+#pragma unroll 4
+    for (int q = r0; q < r1; ++q) {
+        const float2 x = fs.Td[q];
+        if (q == r0 || x.x < Tmin) {
+            kmin = q;
+            Tmin = x.x;
+        }
+        if (x.y > dc && (ia < 0 || x.y < da)) {
+            ia = q;
+            da = x.y;
+        }
+        if (x.y < dc && (ib < 0 || x.y > db)) {
+            ib = q;
+            db = x.y;
+        }
+    }
+    const float ga = ia >= 0 ? da - dc : 100.0f;
+    const float gb = ib >= 0 ? dc - db : 100.0f;
+    const float lag = T - Tmin;
+    const float sk = fs.sd[kmin];
+    f[5] = T / 100.0f;
+    f[6] = fminf(lag, 100.0f) / 10.0f;
+    f[7] = sd;
+    f[8] = fminf(lag / sqrtf(sd * sd + sk * sk + 0.01f), 20.0f) / 5.0f;
+    f[9] = fminf(ga, 100.0f) / 10.0f;
+    f[10] = 1.0f / float(r1 - r0);
+    f[11] = fminf(gb, 100.0f) / 10.0f;
+    const float va = ia >= 0 ? fs.v[ia] : 0.0f, vb = ib >= 0 ? fs.v[ib] : 0.0f, Tb = ib >= 0 ? fs.Td[ib].x : 1.0f;
+    f[12] = (ia >= 0 && vc > va) ? fminf(ga / (vc - va) / T, 2.0f) / 2.0f : 1.0f;
+    f[13] = (ib >= 0 && vb > vc) ? fminf(gb / (vb - vc) / Tb, 2.0f) / 2.0f : 1.0f;
 }
 
 // ------------------------------------------------------------------ forward (tcgen05)
@@ -597,9 +609,9 @@ __global__ void __launch_bounds__(TILE) sg_prep(SgArgs a)
     __shared__ FeatScratch fs;
     const int tid = threadIdx.x, ti = blockIdx.x;
     const SgTile t = a.tiles[ti];
-    build_rowmap(m, a, t, tid, BlockSync{});
+    const int st = build_rowmap(m, a, t, tid);
     float f[KIN];
-    tile_features(f, fs, a, m, tid, BlockSync{});
+    tile_features(f, fs, a, m, tid, st);
     if (a.raw_only) {
 #pragma unroll
         for (int k = RAW; k < KIN; ++k) f[k] = 0.0f;
@@ -618,7 +630,7 @@ __global__ void __launch_bounds__(TILE) sg_prep(SgArgs a)
     }
     if (tid <= t.ns) mt.state_row0[tid] = m.state_row0[tid];
     if (tid < t.ns) mt.state_race[tid] = m.state_race[tid];
-    mt.row_state[tid] = int8_t(m.row_race[tid] >= 0 ? m.row_state[tid] : -1);
+    mt.row_state[tid] = int8_t(st);
 }
 
 template <bool TRAIN>
@@ -1068,12 +1080,6 @@ __global__ void __launch_bounds__(256, 1) sg_backward_chain(SgArgs a, int n_tile
                 }
             }
         }
-        if (tid == 0 && in_ok) {
-            // this tile's term of the b5 gradient; the reduction adds the tiles in order
-            float sdl = 0.0f;
-            for (int q = 0; q < TILE; ++q) sdl += in.dlogit[q];
-            a.b5_part[ti] = sdl;
-        }
         fence_async_smem();
         tc_before_sync();
         __syncthreads();
@@ -1088,6 +1094,19 @@ __global__ void __launch_bounds__(256, 1) sg_backward_chain(SgArgs a, int n_tile
                 tc_mma_d(tmem, smem_desc(sbuf + ks * 256, 128, 16 * 128), smem_desc(w4 + ks * 8192, 4096, 128),
                          idesc_of(2 * H, 0, 1), ks > 0 ? 1u : 0u);
             tc_commit(&sm.mbar);
+        }
+        if (tid == 7 * 32) {
+            // this tile's term of the b5 gradient, while the product runs; the reduction adds the tiles in order
+            float sdl = 0.0f;
+#pragma unroll 8
+            for (int q = 0; q < TILE; q += 4) {
+                const float4 v = *reinterpret_cast<const float4 *>(in.dlogit + q);
+                sdl += v.x;
+                sdl += v.y;
+                sdl += v.z;
+                sdl += v.w;
+            }
+            a.b5_part[ti] = sdl;
         }
         if (block_wait(&sm.mbar, phase, &sm.abort, a)) {
             // dz_g -> bfloat16 over du (the product has read it)
@@ -1201,7 +1220,7 @@ __global__ void __launch_bounds__(256, 1) sg_backward_chain(SgArgs a, int n_tile
 // The weight-gradient kernel streams each tile through shared memory in quarters (32 rows of the
 // reduction) through WG_SLOTS slots: while the tensor cores work on quarter u (and may still be on
 // u - 1), the copies of quarters u + 1 .. u + WG_AHEAD are on their way.
-constexpr int WG_SLOTS = 4;
+constexpr int WG_SLOTS = 5;
 constexpr int WG_AHEAD = WG_SLOTS - 2;                    // quarters fetched ahead of the one in use
 constexpr int WG_ROWS = TILE / 4;                         // rows of one quarter
 constexpr uint32_t WS_QTR = uint32_t(WS_BLOCK / 4);       // 32 rows of a canonical block
@@ -1424,11 +1443,22 @@ __device__ __forceinline__ int param_of_stored(int s)
 
 // gradient = sum over the owning group's blocks of their partials, in block order (b5 is
 // accumulated by the chain kernel and left alone); reads in stored order, writes by parameter
-// The b5 gradient: the tiles' sums of d loss / d logit added in tile order (deterministic).
+// The b5 gradient: the tiles' sums of d loss / d logit added in tile order (deterministic).  A whole warp:
+// it fetches 128 terms at a time, side by side (one thread alone waits for memory every few of them:
+// a step of 4096 states has 430 tiles), and every lane adds them up in order.
 __device__ float b5_gradient(const float *b5_part, int n_tiles)
 {
+    const int lane = threadIdx.x & 31;
     float g = 0.0f;
-    for (int i = 0; i < n_tiles; ++i) g += b5_part[i];
+    for (int i = 0; i < n_tiles; i += 128) {
+        float p[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) p[q] = i + 32 * q + lane < n_tiles ? b5_part[i + 32 * q + lane] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int e = 0; e < 32; ++e) g += __shfl_sync(0xffffffffu, p[q], e);
+    }
     return g;
 }
 
@@ -1436,11 +1466,17 @@ __global__ void sg_reduce_grad(float *grad, const float *partial, int wgroups, c
 {
     pdl_enter();
     const int si = blockIdx.x * blockDim.x + threadIdx.x;
-    if (si == OFF_B5) grad[OFF_B5] = b5_gradient(b5_part, n_tiles);
-    if (si >= N_PARAMS || si == OFF_B5) return;
+    static_assert(OFF_B5 % 32 == 0 && OFF_B5 + 1 == N_PARAMS, "the last parameter has a warp of its own");
+    if (si >= OFF_B5) {
+        if (si >= OFF_B5 + 32) return;
+        const float g = b5_gradient(b5_part, n_tiles);
+        if (si == OFF_B5) grad[OFF_B5] = g;
+        return;
+    }
     const int group = (si >= OFF_W4 && si < OFF_B5) ? 0 : 1;
     const float *src = partial + size_t(group) * wgroups * N_PARAMS + si;
     float s = 0.0f;
+#pragma unroll 16
     for (int c = 0; c < wgroups; ++c) s += src[size_t(c) * N_PARAMS];
     grad[param_of_stored(si)] = s;
 }
@@ -1510,9 +1546,10 @@ __global__ void __launch_bounds__(256) sg_reduce_adam(float *grad, const float *
     int blk = blockIdx.x;
     if (blk >= RA_MATRIX_BLOCKS) {
         const int e = (blk - RA_MATRIX_BLOCKS) * 256 + tid;  // index among the vector parameters
-        if (e > 5 * H) return;
+        static_assert(5 * H % 32 == 0, "b5 has a warp of its own");
+        if (e >= 5 * H + 32) return;
         int pidx;
-        if (e == 5 * H) pidx = OFF_B5;
+        if (e >= 5 * H) pidx = OFF_B5;
         else {
             const int which = e / H, r = e % H;
             const int offs[5] = {OFF_B1, OFF_B2, OFF_B3, OFF_B4, OFF_W5};
@@ -1521,11 +1558,13 @@ __global__ void __launch_bounds__(256) sg_reduce_adam(float *grad, const float *
         float g;
         if (pidx == OFF_B5) {
             g = b5_gradient(b5_part, n_tiles);
+            if (e > 5 * H) return;
             grad[OFF_B5] = g;
         } else {
             const int group = pidx >= OFF_W4 ? 0 : 1;
             const float *src = partial + size_t(group) * wgroups * N_PARAMS + pidx;
             g = 0.0f;
+#pragma unroll 16
             for (int c = 0; c < wgroups; ++c) g += src[size_t(c) * N_PARAMS];
             grad[pidx] = g;
         }
@@ -1544,6 +1583,7 @@ __global__ void __launch_bounds__(256) sg_reduce_adam(float *grad, const float *
         const int si = off + (k0 + y) * H + (j0 + x);  // stored: column k0 + y, row j0 + x
         const float *src = partial + size_t(group) * wgroups * N_PARAMS + si;
         float g = 0.0f;
+#pragma unroll 16
         for (int c = 0; c < wgroups; ++c) g += src[size_t(c) * N_PARAMS];
         tile[y][x] = g;
     }
