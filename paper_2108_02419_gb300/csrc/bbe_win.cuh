@@ -67,8 +67,12 @@ constexpr unsigned kCut = kNone - 1u;  // .. and one whose rollout has run its l
 template <int V, int MODE>
 struct WinStage {
     static constexpr int NS = 32 * V;   // slots per warp
+    // steps of a window, one Philox block: ends are looked for, and rollouts begun, between windows (two
+    // blocks a window halve the ends to handle and waste as much: 31.7 instead of 32.2 ms for 4096 spread
+    // races, 6.8 instead of 5.9 for the short rollouts of a bettor population)
+    static constexpr int W = 4;
     static constexpr int ROW = NS + 2;  // entries per position row: slots, the sentinel, padding to 16 bytes
-    float2 pos[4][ROW];                 // (d, previous step) per slot, one row per step of a block
+    float2 pos[W][ROW];                 // (d, previous step) per slot, one row per step of a window
     float4 pq[32];                      // per competitor: (mu, sigma, P, theta)
     float kr[32];                       // per competitor: kappa (2 rho - 1)
     unsigned pha[32];                   // per competitor: StreamWords::a, the same for all rollouts
@@ -80,8 +84,8 @@ struct WinStage {
     unsigned redo[kContenders ? kRedo + NS : 1];
     unsigned n_redo, rest[2];           // how many; first and end of those not begun for their number
     int wins[MODE == 0 ? 32 : 1];       // wins per competitor in the current work item
-    // by segment base; win mode: the block's least (step, tau) and the first slot that has it; place
-    // mode: the least crossing key not yet placed
+    // by segment base; win mode: the window's least (step, slot) and, among several crossings in that
+    // step, the least tau; place mode: the least crossing key not yet placed
     union {
         unsigned win[2][NS];
         unsigned long long place[NS];
@@ -259,7 +263,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
 {
     constexpr bool PS = WinLean<V>::value;
     using Stage = WinStage<V, MODE>;
-    constexpr int NS = Stage::NS;
+    constexpr int NS = Stage::NS, W = Stage::W;
     constexpr int ROWB = Stage::ROW * int(sizeof(float2));
     constexpr int kSent = NS * int(sizeof(float2));  // byte offset of the sentinel (+inf: no one in front)
     extern __shared__ __align__(16) unsigned char win_smem[];
@@ -278,7 +282,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
     const DevBatch &b = l.b;
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
-        for (int j = 0; j < 4; ++j) st.pos[j][NS] = make_float2(INFINITY, INFINITY);
+        for (int j = 0; j < W; ++j) st.pos[j][NS] = make_float2(INFINITY, INFINITY);
     }
     for (;;) {
         int it = 0;
@@ -535,43 +539,67 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             if (__any_sync(kAll, again)) full_sort(pb, fd, fp);
         };
 
-        // Steps of a Philox block past a crossing, or past the step limit, change nothing that counts (the
-        // rollout ends with the block in any case), so crossings are looked for once a block: positions
-        // only grow, and the block's four rows say which step it was.  (d, S) of that step, for a slot that
-        // has crossed in this block:
-        auto crossing = [&](int v, float &dc, float &Sc) {
-            const int slot = 32 * v + lane;
-            const int J = (st.pos[1][slot].x < L ? 1 : 0) + (st.pos[2][slot].x < L ? 1 : 0) + (st.pos[3][slot].x < L ? 1 : 0);
-            dc = st.pos[J][slot].x;
-            Sc = J < 3 ? st.pos[J + 1][slot].y : pv[v];
+        // Steps of a window past a crossing, or past the step limit, change nothing that counts (the
+        // rollout ends with the window in any case), so crossings are looked for once a window: positions
+        // only grow, and the window's rows say which step it was.  The step in the window, for a slot that
+        // has crossed in it, and its tau = (L - d) / S:
+        auto crossing = [&](int v) {
+            int J = 0;
+#pragma unroll
+            for (int j = 1; j < W; ++j) J += st.pos[j][32 * v + lane].x < L ? 1 : 0;
             return J;
         };
+        auto crossing_tau = [&](int v, int J) {
+            const int slot = 32 * v + lane;
+            const float S = J + 1 < W ? st.pos[J + 1][slot].y : pv[v];
+            return __float_as_uint(__fdiv_rn(__fsub_rn(L, st.pos[J][slot].x), S));
+        };
 
-        // Win mode, the end of a block with a crossing (or, chk, one in which a rollout may have run its
-        // last step): the least key (step, tau) of each segment, then the least slot that has it.  tau =
-        // (L - d) / S is in [0, 2], so its bit pattern less one orders like its value and fits in 30 bits.
+        // Win mode, the end of a window with a crossing (or, chk, one in which a rollout may have run its
+        // last step): the least (step, slot) of each segment.  Where several crossed in that step, the least
+        // tau wins and, among equals, the least slot (tau >= 0, so its bits order like its value); alone,
+        // a crossing needs no tau.
         auto win_end = [&](bool chk, bool (&pend)[V], bool (&again)[V]) {
             unsigned mine[V], kw[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 mine[v] = kNone;
                 if (d[v] >= L) {
-                    float dc, Sc;
-                    const int J = crossing(v, dc, Sc);
-                    if (!chk || int(blk[v]) * 4 - 4 + J < limit) {
-                        const unsigned tau = __float_as_uint(__fdiv_rn(__fsub_rn(L, dc), Sc));
-                        mine[v] = (unsigned(J) << 30) | (max(tau, 1u) - 1u);
+                    const int J = crossing(v);
+                    if (!chk || int(blk[v]) * 4 - W + J < limit) {
+                        mine[v] = unsigned(J) << 8 | unsigned(32 * v + lane);
                         atomicMin(&st.key.win[0][base(v)], mine[v]);
                     }
                 }
                 if (chk && alive(v) && int(blk[v]) * 4 >= limit) atomicMin(&st.key.win[0][base(v)], kCut);
             }
             __syncwarp();
+            bool tie = false;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 kw[v] = alive(v) ? st.key.win[0][base(v)] : kNone;
                 pend[v] = kw[v] != kNone;
-                if (pend[v] && mine[v] == kw[v]) atomicMin(&st.key.win[1][base(v)], unsigned(32 * v + lane));
+                tie |= mine[v] > kw[v] && (mine[v] >> 8) == (kw[v] >> 8);
+            }
+            if (__any_sync(kAll, tie)) {
+                unsigned tau[V];
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    tau[v] = kNone;
+                    if (mine[v] != kNone && (mine[v] >> 8) == (kw[v] >> 8)) {
+                        tau[v] = crossing_tau(v, int(mine[v] >> 8));
+                        atomicMin(&st.key.win[1][base(v)], tau[v]);
+                    }
+                    if (pend[v] && kw[v] != kCut && 32 * v + lane == base(v)) st.key.win[0][base(v)] = kw[v] | 255u;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    if (tau[v] != kNone && tau[v] == st.key.win[1][base(v)]) atomicMin(&st.key.win[0][base(v)], mine[v]);
+                __syncwarp();
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    if (pend[v]) kw[v] = st.key.win[0][base(v)];
             }
             __syncwarp();
 #pragma unroll
@@ -586,14 +614,14 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                         again[v] = true;
                     }
                 } else {
-                    atomicAdd(&st.wins[BBE_INDEX(int(st.key.win[1][slot]) - slot, 32, l.status)], 1);
-                    steps += (unsigned long long)(blk[v] * 4u - 3u + (kw[v] >> 30));
+                    atomicAdd(&st.wins[BBE_INDEX(int(kw[v] & 255u) - slot, 32, l.status)], 1);
+                    steps += (unsigned long long)(blk[v] * 4u - unsigned(W - 1) + (kw[v] >> 8));
                 }
                 st.key.win[0][slot] = st.key.win[1][slot] = kNone;
             }
         };
 
-        // Place mode, the same: the block's crossings of each segment take the next places one at a
+        // Place mode, the same: the window's crossings of each segment take the next places one at a
         // time in key order (step, tau, slot), and a segment whose K-th place is filled ends its
         // rollout; one stopped at max_steps that did not end earlier counts for nobody.
         auto place_end = [&](bool chk, bool (&pend)[V], bool (&again)[V]) {
@@ -606,12 +634,10 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 sb[v] = base(v);
                 fk[v] = kNoKey;
                 if (d[v] >= L && st.pos[0][slot].x < L) {
-                    float dc, Sc;
-                    const int J = crossing(v, dc, Sc);
-                    if (!chk || int(blk[v]) * 4 - 4 + J < limit) {
-                        const float tau = __fdiv_rn(__fsub_rn(L, dc), Sc);
+                    const int J = crossing(v);
+                    if (!chk || int(blk[v]) * 4 - W + J < limit) {
                         fk[v] = (static_cast<unsigned long long>(J) << 40) |
-                                (static_cast<unsigned long long>(__float_as_uint(tau)) << 8) | unsigned(slot);
+                                (static_cast<unsigned long long>(crossing_tau(v, J)) << 8) | unsigned(slot);
                         more = true;
                     }
                 }
@@ -648,7 +674,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 const int slot = 32 * v + lane;
                 const unsigned filled = pl_n[sb[v]];
                 if (filled >= kPlaced) {
-                    if (slot == sb[v]) steps += (unsigned long long)(blk[v] * 4u - 3u + filled - kPlaced);
+                    if (slot == sb[v]) steps += (unsigned long long)(blk[v] * 4u - unsigned(W - 1) + filled - kPlaced);
                     pend[v] = true;
                 } else if (chk && int(blk[v]) * 4 >= limit) {
                     if (limit >= l.max_steps) {
@@ -699,7 +725,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             __syncwarp();
         };
 
-        // One step of every slot: step j0 + J of the Philox block, with the normal z[v][J].
+        // One step of every slot: step j0 + J of the window, with the normal z[v][J].
         int j0 = 0;
         auto step = [&](auto Jc, const float (&z)[V][4]) {
             constexpr int J = decltype(Jc)::value;
@@ -747,35 +773,38 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             }
         };
 
-        // blocks before one at whose end a rollout can have run `limit` steps: no slot is further into
-        // its rollout than the blocks the work item has run, so a warp-uniform count-down rules the
+        // windows before one at whose end a rollout can have run `limit` steps: no slot is further into
+        // its rollout than the windows the work item has run, so a warp-uniform count-down rules the
         // check out in all but the longest items
-        unsigned left = unsigned(max(limit, 1) - 1) / 4u;
+        unsigned left = unsigned(max(limit, 1) - 1) / unsigned(W);
         for (bool live = k_count > 0u; live;) {
-            // the block's normals: one Philox4x32-10 output per slot, counter (k, t >> 2, c, race)
+            // a block's normals: one Philox4x32-10 output per slot, counter (k, t >> 2, c, race)
             float z[V][4];
+            auto draw = [&]() {
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-                draw_block<DIST>(st.ph[32 * v + lane], PS ? st.pha[kra[v] - st.kr] : pha[v], blk[v], l.round_key, z[v]);
+                for (int v = 0; v < V; ++v)
+                    draw_block<DIST>(st.ph[32 * v + lane], PS ? st.pha[kra[v] - st.kr] : pha[v], blk[v], l.round_key, z[v]);
+            };
             if constexpr (MODE == 0) {
-                // two copies of the step, run twice (the second time with the block's other two
-                // normals): with four, the steps and their repairs overflow the instruction cache where
+                // two copies of the step, run twice (the second time with the block's other two normals): with four, the steps and their repairs overflow the instruction cache where
                 // overtakes are frequent (700 bunched races of 13: 15.3 instead of 14.6 ms; spread races
                 // without overtakes lose 1 to 2 %)
 #pragma unroll 1
-                for (;;) {
+                for (j0 = 0; j0 < W; j0 += 2) {
+                    if (j0 == 0) {
+                        draw();
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < V; ++v) {
+                            z[v][0] = z[v][2];
+                            z[v][1] = z[v][3];
+                        }
+                    }
                     step(std::integral_constant<int, 0>{}, z);
                     step(std::integral_constant<int, 1>{}, z);
-                    if (j0 != 0) break;
-                    j0 = 2;
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        z[v][0] = z[v][2];
-                        z[v][1] = z[v][3];
-                    }
                 }
-                j0 = 0;
             } else {
+                draw();
                 step(std::integral_constant<int, 0>{}, z);
                 step(std::integral_constant<int, 1>{}, z);
                 step(std::integral_constant<int, 2>{}, z);
@@ -786,7 +815,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             bool event = false;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                ++blk[v];
+                blk[v] += unsigned(W / 4);
                 event |= d[v] >= L && (MODE == 0 || st.pos[0][32 * v + lane].x < L);
             }
             if (chk) {
