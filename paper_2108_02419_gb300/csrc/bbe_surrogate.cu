@@ -351,6 +351,15 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(H >> 3) << 17) | (uint32_t(TILE >> 4) << 24);
 constexpr uint32_t kIdescBmn = kIdesc | (1u << 16);
 
+// The descriptor of an operand `bytes` further on in shared memory (a multiple of 16; the start
+// address stays within its 14-bit field, so one 32-bit addition does).  A layer's products differ from one
+// another by this only; building each descriptor from its address kept the issuing thread behind the tensor
+// cores.
+__device__ __forceinline__ uint64_t desc_add(uint64_t d, uint32_t bytes)
+{
+    return (d & 0xFFFFFFFF00000000ull) | uint64_t(uint32_t(d) + (bytes >> 4));
+}
+
 // D (+)= A . B^T with A and B in shared memory
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t ad, uint64_t bd, uint32_t accumulate)
 {
@@ -416,6 +425,20 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// A thread's biases of 32 columns, fetched while the product whose accumulators they go with still runs.
+struct Bias32 {
+    float2 b[16];
+    __device__ __forceinline__ void load(const float *bias)
+    {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = *reinterpret_cast<const float4 *>(bias + 4 * i);
+            b[2 * i] = make_float2(v.x, v.y);
+            b[2 * i + 1] = make_float2(v.z, v.w);
+        }
+    }
+};
+
 // bfloat16 pair {relu(lo), relu(hi)} rounded to nearest (lo in the low half)
 __device__ __forceinline__ uint32_t relu_bf16x2(float lo, float hi)
 {
@@ -441,7 +464,7 @@ __device__ __forceinline__ uint32_t pos_bits(uint32_t pk)
 
 // bias + ReLU -> bfloat16 into the canonical activation tile (and, TRAIN, the workspace block and mask)
 template <bool TRAIN>
-__device__ __forceinline__ void tc_epilogue_relu(uint32_t taddr, const float *bias, unsigned char *act, int row,
+__device__ __forceinline__ void tc_epilogue_relu(uint32_t taddr, const float *bias, Bias32 &b, unsigned char *act, int row,
                                                  unsigned char *ws_blk, uint32_t *ws_mask, int c0)
 {
     unsigned char *arow = act + act_row(row);
@@ -458,13 +481,15 @@ __device__ __forceinline__ void tc_epilogue_relu(uint32_t taddr, const float *bi
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int j = q * 8 + 2 * e;
-                pk[e] = relu_bf16x2(__uint_as_float(r[j]) + bias[cb + j], __uint_as_float(r[j + 1]) + bias[cb + j + 1]);
+                const float2 z = __fadd2_rn(make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), b.b[j / 2]);
+                pk[e] = relu_bf16x2(z.x, z.y);
                 if (TRAIN) bits |= pos_bits(pk[e]) << j;
             }
             const uint4 v = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             *reinterpret_cast<uint4 *>(arow + ((cb >> 3) + q) * 128) = v;
             if (TRAIN) *reinterpret_cast<uint4 *>(ws_blk + act_row(row) + ((cb >> 3) + q) * 128) = v;
         }
+        if (cb == c0) b.load(bias + c0 + 32);
         if (TRAIN) ws_mask[row * 4 + (cb >> 5)] = bits;
     }
 }
@@ -472,7 +497,7 @@ __device__ __forceinline__ void tc_epilogue_relu(uint32_t taddr, const float *bi
 // head: u = bfloat16(relu(acc + b4)) (workspace block and mask when training); returns this
 // half's w5 . u
 template <bool TRAIN>
-__device__ __forceinline__ float tc_epilogue_head(uint32_t taddr, const float *b4, const float *w5, int row,
+__device__ __forceinline__ float tc_epilogue_head(uint32_t taddr, const float *b4, Bias32 &b, const float *w5, int row,
                                                   unsigned char *ws_blk, uint32_t *ws_mask, int c0)
 {
     float s = 0.0f;
@@ -489,7 +514,8 @@ __device__ __forceinline__ float tc_epilogue_head(uint32_t taddr, const float *b
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int j = q * 8 + 2 * e;
-                pk[e] = relu_bf16x2(__uint_as_float(r[j]) + b4[cb + j], __uint_as_float(r[j + 1]) + b4[cb + j + 1]);
+                const float2 z = __fadd2_rn(make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), b.b[j / 2]);
+                pk[e] = relu_bf16x2(z.x, z.y);
                 s += __uint_as_float(pk[e] << 16) * w5[cb + j] + __uint_as_float(pk[e] & 0xFFFF0000u) * w5[cb + j + 1];
                 if (TRAIN) bits |= pos_bits(pk[e]) << j;
             }
@@ -497,6 +523,7 @@ __device__ __forceinline__ float tc_epilogue_head(uint32_t taddr, const float *b
                 *reinterpret_cast<uint4 *>(ws_blk + act_row(row) + ((cb >> 3) + q) * 128) =
                     make_uint4(pk[0], pk[1], pk[2], pk[3]);
         }
+        if (cb == c0) b.load(b4 + c0 + 32);
         if (TRAIN) ws_mask[row * 4 + (cb >> 5)] = bits;
     }
     return s;
@@ -687,6 +714,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sg_forward_tc(SgArgs a, int n_t
     const uint32_t lane_off = uint32_t((warp & 3) * 32) << 16;
     const uint32_t td = tmem + lane_off, ts = tmem + H + lane_off, tg = tmem + H + H / 2 + lane_off;
     const uint32_t sact = smem_addr(P.act), sw = smem_addr(sm.w);
+    // operands: activations (and the same tile read MN-major), W2 (W3 behind it), W4
+    const uint64_t dact = smem_desc(sact, 128, 16 * 128), dact_t = smem_desc(sact, 2048, 128);
+    const uint64_t dw2 = smem_desc(sw + WC_W2 * 2, 128, 16 * 128), dw4 = smem_desc(sw + WC_W4 * 2, 128, 32 * 128);
     const int row = (warp & 3) * 32 + lane;  // tile row of this thread = its TMEM lane
     const int c0 = ch * (H / 2);             // first accumulator column of this thread
     uint32_t phase = 0;
@@ -740,8 +770,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sg_forward_tc(SgArgs a, int n_t
             tc_store_pool_row(ts, r0, r1, c0);
             tmem_wait_st();
         }
+        Bias32 bias;
+        bias.load(sm.bias[0] + c0);
         if (group_wait(sm, p, phase, a))
-            tc_epilogue_relu<TRAIN>(td, sm.bias[0], P.act, row, ws ? ws + WS_H1 : nullptr, wsm, c0);
+            tc_epilogue_relu<TRAIN>(td, sm.bias[0], bias, P.act, row, ws ? ws + WS_H1 : nullptr, wsm, c0);
         fence_async_smem();
         tc_before_sync();
         sync();
@@ -751,15 +783,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sg_forward_tc(SgArgs a, int n_t
         for (int l = 1; l <= 2; ++l) {
             if (pt == 0) {
                 tc_after_sync();
-                const uint32_t wl = sw + uint32_t(l == 1 ? WC_W2 : WC_W3) * 2;
+                const uint64_t dw = l == 1 ? dw2 : desc_add(dw2, (WC_W3 - WC_W2) * 2);
 #pragma unroll
                 for (int ks = 0; ks < H / 16; ++ks)
-                    tc_mma(tmem, smem_desc(sact + ks * 256, 128, 16 * 128), smem_desc(wl + ks * 256, 128, 16 * 128),
-                           ks > 0 ? 1u : 0u);
+                    tc_mma(tmem, desc_add(dact, ks * 256), desc_add(dw, ks * 256), ks > 0 ? 1u : 0u);
                 tc_commit(&sm.mbar[p]);
             }
+            bias.load(sm.bias[l] + c0);
             if (group_wait(sm, p, phase, a))
-                tc_epilogue_relu<TRAIN>(td, sm.bias[l], P.act, row, ws ? ws + WS_H1 + l * WS_BLOCK : nullptr,
+                tc_epilogue_relu<TRAIN>(td, sm.bias[l], bias, P.act, row, ws ? ws + WS_H1 + l * WS_BLOCK : nullptr,
                                  wsm ? wsm + l * (WS_MASK / 4) : nullptr, c0);
             fence_async_smem();
             tc_before_sync();
@@ -774,7 +806,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sg_forward_tc(SgArgs a, int n_t
             tc_after_sync();
 #pragma unroll
             for (int ks = 0; ks < TILE / 16; ++ks)
-                tc_mma_ta(tmem, tmem + H + ks * 8, smem_desc(sact + ks * 4096, 2048, 128), kIdescBmn, ks > 0 ? 1u : 0u);
+                tc_mma_ta(tmem, tmem + H + ks * 8, desc_add(dact_t, ks * 4096), kIdescBmn, ks > 0 ? 1u : 0u);
             tc_commit(&sm.mbar[p]);
         }
         if (group_wait(sm, p, phase, a)) tc_epilogue_pool<TRAIN>(td, tg, inv_n, row, ws ? ws + WS_G : nullptr, c0);
@@ -788,17 +820,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sg_forward_tc(SgArgs a, int n_t
             tc_after_sync();
 #pragma unroll
             for (int ks = 0; ks < H / 16; ++ks)
-                tc_mma(tmem, smem_desc(sact + ks * 256, 128, 16 * 128), smem_desc(sw + WC_W4 * 2 + ks * 256, 128, 32 * 128),
-                       ks > 0 ? 1u : 0u);
+                tc_mma(tmem, desc_add(dact, ks * 256), desc_add(dw4, ks * 256), ks > 0 ? 1u : 0u);
 #pragma unroll
             for (int ks = 0; ks < H / 16; ++ks)
-                tc_mma_ta(tmem, tmem + H + H / 2 + ks * 8, smem_desc(sw + WC_W4 * 2 + (H / 16 + ks) * 256, 128, 32 * 128),
-                          kIdesc, 1u);
+                tc_mma_ta(tmem, tmem + H + H / 2 + ks * 8, desc_add(dw4, (H / 16 + ks) * 256), kIdesc, 1u);
             tc_commit(&sm.mbar[p]);
         }
+        bias.load(sm.bias[3] + c0);
         if (group_wait(sm, p, phase, a))
             P.logit_part[ch][row] =
-                tc_epilogue_head<TRAIN>(td, sm.bias[3], sm.w5, row, ws ? ws + WS_U : nullptr, wsm ? wsm + 3 * (WS_MASK / 4) : nullptr,
+                tc_epilogue_head<TRAIN>(td, sm.bias[3], bias, sm.w5, row, ws ? ws + WS_U : nullptr, wsm ? wsm + 3 * (WS_MASK / 4) : nullptr,
                                  c0);
         fence_async_smem();
         tc_before_sync();
