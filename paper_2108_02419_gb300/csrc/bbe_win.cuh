@@ -146,11 +146,11 @@ __device__ __forceinline__ float warp_max(float v)
 //
 // H is an estimate of the K-th finish with a margin of three standard deviations; the few rollouts
 // that are still running after H steps are run again with everybody.
-// x: 3 n floats of scratch.  Called by the whole warp; lane c < n holds competitor c.
+// x: 3 n floats of scratch; slots: of the warp.  Called by the whole warp; lane c < n holds competitor c.
 template <int DIST, int LAW>
 __device__ __forceinline__ unsigned contender_mask(float *x, int n, int lane, float d, float mu, float sigma, float P,
                                                    float kr, float prev, float theta, float L, float invL, float t0,
-                                                   float invT, int K, int &H)
+                                                   float invT, int K, int slots, int &H)
 {
     const bool on = lane < n;
     const unsigned everybody = kAll >> (32 - n);
@@ -175,8 +175,9 @@ __device__ __forceinline__ unsigned contender_mask(float *x, int n, int lane, fl
     const float Rlo = 1.0f + kr * (lo - 0.5f);
     const float R = 1.00001f * fmaxf(Rlo, 1.0f + kr * (end - 0.5f));
     const float F = 1.0001f * fmaxf(warp_max(on ? fmaxf(prev, R * P * (mu + zmax * sigma)) : 0.0f), kStepFloor);
-    const float dmin = warp_min(on ? d : INFINITY), goal = 0.9999f * L;
-    if (!(goal - float(H) * F > dmin)) return everybody;  // not even at the free pace
+    const float goal = 0.9999f * L;
+    // not even at the free pace would there be room for more segments
+    if (slots / max(1, __popc(__ballot_sync(kAll, on && !(goal - float(H) * F > d)))) <= slots / n) return everybody;
     const float lambda = 1.00001f * fmaxf(warp_max(on ? R : 0.0f), 1.0f);  // anywhere
     // from here on lane i holds rank i
     if (on) {
@@ -337,10 +338,14 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         // that makes room for more segments
         unsigned keep = kAll >> (32 - n_race);
         int limit = l.max_steps;  // a rollout that reaches it ends undecided
-        if (Stage::kContenders && pass == kFirst && l.contenders && K < n_race) {
+        // Finding them takes about as long as one rollout of every segment, so only where a warp runs at
+        // least eight (2010 races of 10 to the sixth, 55 rollouts each: 709 us with them, 531 without).
+        if (Stage::kContenders && pass == kFirst && l.contenders && K < n_race &&
+            min(min(Rr, int64_t(l.per_lane) * (NS / n_race)), int64_t(max(l.most, w.k_count))) >= 8 * (NS / n_race)) {
             int H = 0;
             const unsigned front = contender_mask<DIST, LAW>(reinterpret_cast<float *>(st.ph), n_race, lane, my_d0, my_mu,
-                                                             my_sg, my_P, my_kr, my_pv, my_th, L, invL, t0r, invTr, K, H);
+                                                             my_sg, my_P, my_kr, my_pv, my_th, L, invL, t0r, invTr, K, NS,
+                                                             H);
             const int nf = __popc(front);
             if (nf >= K && (l.seg_cap > 0 ? min(NS / nf, l.seg_cap) > min(NS / n_race, l.seg_cap) : NS / nf > NS / n_race)) {
                 keep = front;
