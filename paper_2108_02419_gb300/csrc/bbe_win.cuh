@@ -21,8 +21,8 @@
 // per slot (from words kept per rollout, StreamWords) and both of its Box-Muller pairs, then runs
 // four steps whose normals are registers chosen at compile time.  Every rollout starts on a block boundary (a
 // segment that finishes waits for the next one; the counter of step t is t >> 2 in any case).
-// A finished segment takes its next rollout index from a per-warp counter, so the segments of
-// a work item stay busy until its rollouts run out.
+// A finished segment takes the warp's next rollout index, so the segments of a work item stay busy until
+// its rollouts run out.
 //
 // Who is advanced.  Only the competitors that can matter to the first finish, or the first K, are
 // (contender_mask); they take the slots, so a warp has room for more segments.  A work item is a
