@@ -12,6 +12,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <optional>
 #include <string>
 #include <vector>
 
@@ -222,7 +223,9 @@ __global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, i
     items[i] = bbe::WorkItem{race, tickets ? r.k0 : r.k0 + j * r.chunk, r.chunk, 0};
 }
 
-bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
+// on: the stream to build the list on, any handle, 0 (the default stream) included; none: the batch's
+// own free stream, for the calls that are given no stream.  Waits for it before returning.
+bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullopt)
 {
     const int32_t n_rec = b->n_races / b->reps;  // host records, each of `reps` equal races
     // Per race: full chunks of `chunk` rollouts (all of one cost) and a remainder.  The list puts
@@ -334,15 +337,12 @@ bbe_status build_items(bbe_batch *b, cudaStream_t upload = nullptr)
         for (int g = 0; g < kGroups; ++g)
             if (!plans[g].empty()) full = int32_t(std::max<int64_t>(1, plans[g][0].full));
 
-    // the new list is in place before the call returns (made on `upload`, the staging call's
-    // stream, else on the batch's free stream); the old one is freed behind this batch's work
+    // the new list is in place before the call returns; the old one is freed behind this batch's work
     // that may still read it
     bbe::WorkItem *fresh = nullptr;
     ItemRun *d_runs = nullptr;
-    if (!upload) {
-        BBE_CUDA_TRY(ensure_free_stream(b));
-        upload = b->free_stream;
-    }
+    if (!on) BBE_CUDA_TRY(ensure_free_stream(b));
+    const cudaStream_t upload = on ? *on : b->free_stream;
     BBE_CUDA_TRY(pool_alloc(reinterpret_cast<void **>(&fresh), std::max<size_t>(1, size_t(listed)) * sizeof(bbe::WorkItem), upload));
     if (!runs.empty()) {
         BBE_CUDA_TRY(pool_alloc(reinterpret_cast<void **>(&d_runs), runs.size() * sizeof(ItemRun), upload));
@@ -674,6 +674,7 @@ bbe_status bbe::stage_repeated(bbe_batch **out, int32_t n_rec, int32_t reps, int
     b->h_theta = std::move(theta);
     b->h_prev = std::move(prev);
     auto fail = [&](bbe_status code) {
+        cudaStreamSynchronize(s);  // copies from `rec` and into the batch may be queued
         bbe_destroy_batch(b);
         return code;
     };
@@ -779,7 +780,8 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
     std::vector<float> &h_sigma = b->h_sigma, &h_rho = b->h_rho, &h_P = b->h_P, &h_theta = b->h_theta,
                        &h_prev = b->h_prev;
     auto fail = [&](bbe_status code) {
-        bbe_destroy_batch(b);  // frees whatever was allocated so far
+        cudaStreamSynchronize(s);  // copies from the arrays here and into the batch may be queued
+        bbe_destroy_batch(b);      // frees whatever was allocated so far
         return code;
     };
     if ((st = copy_in(b->h_L.data(), track_len, n_races * sizeof(float), s, "track_len", &pending)) ||
