@@ -1253,8 +1253,22 @@ __global__ void __launch_bounds__(256, 1) sg_backward_chain(SgArgs a, int n_tile
 // u - 1), the copies of quarters u + 1 .. u + WG_AHEAD are on their way.
 constexpr int WG_SLOTS = 5;
 constexpr int WG_AHEAD = WG_SLOTS - 2;                    // quarters fetched ahead of the one in use
-constexpr int WG_ROWS = TILE / 4;                         // rows of one quarter
+constexpr int WG_PARTS = 4;                               // quarters of a tile
+constexpr int WG_ROWS = TILE / WG_PARTS;                  // rows of one quarter
 constexpr uint32_t WS_QTR = uint32_t(WS_BLOCK / 4);       // 32 rows of a canonical block
+
+// Which products are done when.  Quarter u's iteration waits for the product of quarter u - WG_LAG (and so for
+// all before it: products finish in order) whether or not a copy follows, because two buffers are
+// written after that wait:
+//   the slot of quarter u + WG_AHEAD, last read by the product of quarter u + WG_AHEAD - WG_SLOTS;
+//   the d logit columns of quarter u's part (`dls` has one block of columns a part, not a slot), last
+//   read by the product of quarter u - WG_PARTS.
+// (With the wait tied to the copy, the last WG_AHEAD quarters rewrote columns that a product of the tile
+// before might still read.)  The waits take each slot's products in order, one phase at a time; the last
+// WG_LAG products are left for the end.
+constexpr int WG_LAG = WG_SLOTS - WG_AHEAD;
+static_assert(WG_AHEAD >= 1 && WG_LAG >= 1, "a copy ahead of, and a product behind, the quarter in use");
+static_assert(WG_LAG <= WG_PARTS, "a part's d logit columns are rewritten after the product that read them last");
 
 struct BwSmem {
     // WG_SLOTS slots, each one quarter of a tile: group 0 du, h3, g, u; group 1 da3, h2, da2, h1,
@@ -1318,7 +1332,7 @@ __global__ void __launch_bounds__(128, 1) sg_backward_wgrad(SgArgs a, int n_tile
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // constant operands: ones in row 0, zeros elsewhere (rows 0 and 1 of dls are rewritten per quarter)
+    // constant operands: ones in row 0, zeros elsewhere (rows 0 and 1 of dls are rewritten per quarter, see WG_LAG)
     for (int i = tid; i < 16 * TILE; i += 128) {
         const int n = i / TILE, kk = i - n * TILE;
         *reinterpret_cast<bf16 *>(sm.ones + nk_off(n, kk)) = __float2bfloat16_rn(n == 0 ? 1.0f : 0.0f);
@@ -1330,6 +1344,7 @@ __global__ void __launch_bounds__(128, 1) sg_backward_wgrad(SgArgs a, int n_tile
     tc_after_sync();
     const uint32_t tmem = sm.tmem_base;
     const uint32_t sones = smem_addr(sm.ones), sdls = smem_addr(sm.dls);
+    static_assert(WG_PARTS == 4, "u & 3, u >> 2");
     // this block's quarters: u = 0 .. n_q-1 is quarter (u & 3) of its (u >> 2)-th tile
     const int my_tiles = cta < n_tiles ? (n_tiles - 1 - cta) / a.wgroups + 1 : 0;
     const int n_q = 4 * my_tiles;
@@ -1355,15 +1370,13 @@ __global__ void __launch_bounds__(128, 1) sg_backward_wgrad(SgArgs a, int n_tile
     int done_q = 0;
     for (int u = 0; u < n_q; ++u) {
         const int slot = u % WG_SLOTS, part = u & 3;
-        // fetch quarter u + WG_AHEAD into the slot of quarter u + WG_AHEAD - WG_SLOTS, once that
-        // quarter's product has finished (the product of u - 1 may still be running)
+        // the product of quarter u - WG_LAG has finished (that of u - 1 may still be running): its slot
+        // takes quarter u + WG_AHEAD, and this part's d logit columns may be rewritten
         const int nxt = u + WG_AHEAD, nslot = nxt % WG_SLOTS;
-        if (nxt < n_q) {
-            if (nxt >= WG_SLOTS && !wait_slot(&sm.mbar_mma[nslot], mma_bits, nslot)) break;
-            if (tid == 0) {
-                load_wgrad_quarter(sm, nslot, group, cta + (nxt >> 2) * a.wgroups, nxt & 3, a);
-                note_copy(nslot);
-            }
+        if (u >= WG_LAG && !wait_slot(&sm.mbar_mma[nslot], mma_bits, nslot)) break;
+        if (nxt < n_q && tid == 0) {
+            load_wgrad_quarter(sm, nslot, group, cta + (nxt >> 2) * a.wgroups, nxt & 3, a);
+            note_copy(nslot);
         }
         if (!wait_slot(&sm.mbar_in[slot], in_bits, slot)) break;
         pend_bits &= ~(1u << slot);
