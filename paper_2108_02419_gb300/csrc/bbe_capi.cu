@@ -719,7 +719,7 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
                             const int64_t *rollouts, const float *pos, const float *mu, const float *sigma,
                             const float *resp, const float *pref, const float *theta, const float *prev_step,
                             uint64_t seed, bbe_dist dist, uint32_t race_id0, const int32_t *race_ids,
-                            cudaStream_t s)
+                            cudaStream_t s, bool in_order)
 {
     if (!out) {
         set_error("out is NULL");
@@ -734,6 +734,8 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
         set_error("unknown distribution");
         return BBE_ERR_ARG;
     }
+    // host memory is read by the host itself, so what the stream still has to write there comes first
+    if (in_order) BBE_CUDA_TRY(cudaStreamSynchronize(s));
     std::vector<int32_t> off(size_t(n_races) + 1);
     bool pending = false;  // a copy from device memory is under way
     bbe_status st = copy_in(off.data(), race_off, off.size() * sizeof(int32_t), s, "race_off", &pending);
@@ -893,7 +895,7 @@ bbe_status bbe_race_init(bbe_batch **out, int32_t n_races, const int32_t *race_o
                          uint64_t seed, bbe_dist dist, uint32_t race_id0, void *cuda_stream)
 {
     return bbe::stage_batch(out, n_races, race_off, track_len, rollouts, pos, mu, sigma, resp, pref, theta,
-                            prev_step, seed, dist, race_id0, nullptr, as_stream(cuda_stream));
+                            prev_step, seed, dist, race_id0, nullptr, as_stream(cuda_stream), true);
 }
 
 bbe_status bbe_rollout_batch(bbe_batch *b, int32_t *win_counts, int64_t *steps_total, void *cuda_stream)

@@ -240,12 +240,13 @@ struct bbe_batch {
 
 
 namespace bbe {
-// bbe_race_init with an optional explicit stream id per race (host array, may be null).
+// bbe_race_init with an optional explicit stream id per race (host array, may be null).  in_order: the
+// arrays are a caller's, and those in host memory hold their values when the stream's work so far is done.
 bbe_status stage_batch(bbe_batch **out, int32_t n_races, const int32_t *race_off, const float *track_len,
                        const int64_t *rollouts, const float *pos, const float *mu, const float *sigma,
                        const float *resp, const float *pref, const float *theta, const float *prev_step,
                        uint64_t seed, bbe_dist dist, uint32_t race_id0, const int32_t *race_ids,
-                       cudaStream_t stream);
+                       cudaStream_t stream, bool in_order = false);
 // Run rollouts k0[r] .. k0[r] + R[r] - 1 of race r instead of 0 .. R[r] - 1 (host array;
 // k0[r] + R[r] <= 2^31 - 1).  The counts of such a batch added to those of rollouts
 // 0 .. k0[r] - 1 equal the counts of one batch of k0[r] + R[r] rollouts.

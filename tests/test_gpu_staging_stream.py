@@ -86,3 +86,29 @@ def test_a_snapshot_batch_is_in_place_when_the_call_returns():
     want_c, want_s, _ = oracle.batch_counts(one)
     assert np.array_equal(got_c, want_c)
     assert np.array_equal(got_s, want_s)
+
+
+def test_host_arrays_are_read_when_the_stream_has_written_them():
+    # every array in pinned memory, filled by copies that are still queued when the call is made
+    from paper_2108_02419_gb300 import bbe
+
+    rb = small(7, 40)
+    rb.prev0 = (rb.mu * rb.P).astype(np.float32)
+    s = torch.cuda.Stream()
+    host = [np.ascontiguousarray(a) for a in (rb.race_off, rb.L, rb.rollouts, rb.d0, rb.mu, rb.sigma, rb.rho, rb.P, rb.theta,
+                                             rb.prev0)]
+    there = [torch.from_numpy(a).cuda() for a in host]
+    here = [torch.from_numpy(np.zeros_like(a)).pin_memory() for a in host]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        busy()
+        for h, t in zip(here, there):
+            h.copy_(t, non_blocking=True)
+    h = bbe.bbe_race_init(rb.n_races, *here[:7], here[7], here[8], here[9], rb.seed, rb.dist, rb.race_id0, s)
+    try:
+        got_c, got_s = rolled(h, rb, s)
+    finally:
+        bbe.bbe_destroy_batch(h)
+    want_c, want_s, _ = oracle.batch_counts(rb)
+    assert np.array_equal(got_c, want_c)
+    assert np.array_equal(got_s, want_s)
