@@ -383,6 +383,10 @@ bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *ste
     l.per_lane = b->per_lane;
     l.most = b->most;
     l.contenders = b->tickets ? 1 : 0;
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    if (b->always_contenders) l.contenders = 2;
+    l.seen = b->d_seen;
+#endif
     l.counts = counts;
     l.steps = reinterpret_cast<unsigned long long *>(steps);
     l.status = b->d_status;
@@ -400,6 +404,10 @@ bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *ste
 // Queue heads, status and, behind them, the races' ticket counters: one range.
 cudaError_t reset_queue(const bbe_batch *b, cudaStream_t s)
 {
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    const cudaError_t e = cudaMemsetAsync(b->d_seen, 0, bbe::kSeen * sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+#endif
     return cudaMemsetAsync(b->d_queue, 0, (kGroups + 1 + (b->tickets ? size_t(b->n_races) : 0)) * sizeof(int32_t), s);
 }
 
@@ -548,7 +556,7 @@ bbe_status make_arena(bbe_batch *b, Arena &A, cudaStream_t s)
     auto add = [&](size_t n) { bytes += (n + 255) / 256 * 256; };
     add((n_races + 1) * 4); add(n_races * 4); add(n_races * 8); add(nt * 4); add(n_races * 4);
     for (int i = 0; i < 7; ++i) add(nt * 4);
-    add((kGroups + 1 + n_races) * 4);
+    add((kGroups + 1 + n_races + bbe::kSeen) * 4);
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e == cudaSuccess) e = pool_alloc(&b->arena, bytes, s);
@@ -564,9 +572,12 @@ bbe_status make_arena(bbe_batch *b, Arena &A, cudaStream_t s)
     A.cr = carve<int32_t>(p, nt);
     A.ids = carve<int32_t>(p, n_races);
     for (float **q : {&A.d0, &A.mu, &A.sigma, &A.rho, &A.P, &A.theta, &A.prev}) *q = carve<float>(p, nt);
-    b->d_queue = carve<int32_t>(p, kGroups + 1 + n_races);
+    b->d_queue = carve<int32_t>(p, kGroups + 1 + n_races + bbe::kSeen);
     b->d_status = b->d_queue + kGroups;
     b->d_next = b->d_status + 1;
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    b->d_seen = b->d_next + n_races;
+#endif
     return BBE_OK;
 }
 
@@ -1534,6 +1545,25 @@ bbe_status bbe_batch_launches(const bbe_batch *b, int32_t *kernels_per_pass)
     *kernels_per_pass = k;
     return BBE_OK;
 }
+
+#if defined(BBE_CHECKED) && BBE_CHECKED
+// Checked build only.  always: the batch's passes look for contenders whatever that costs.
+BBE_API bbe_status bbe_checked_contenders(bbe_batch *b, int32_t always)
+{
+    b->always_contenders = always != 0;
+    free_graph(b);
+    return BBE_OK;
+}
+
+// Checked build only: seen[kSeen] of the batch's last pass (waits for the stream).
+BBE_API bbe_status bbe_checked_seen(const bbe_batch *b, int32_t *seen, void *cuda_stream)
+{
+    cudaStream_t s = as_stream(cuda_stream);
+    BBE_CUDA_TRY(cudaMemcpyAsync(seen, b->d_seen, bbe::kSeen * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBE_CUDA_TRY(cudaStreamSynchronize(s));
+    return BBE_OK;
+}
+#endif
 
 void bbe_destroy_batch(bbe_batch *b)
 {

@@ -78,7 +78,22 @@ struct RolloutLaunch {
     unsigned long long *hist_keys;  // place-count kernel, or null: finishing-order hash tables (keys)
     int32_t *hist_counts;           // the count beside each key
     const int64_t *hist_off;        // [n_races + 1]: each race's table (a power of two of entries)
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    int32_t *seen;           // [kSeen] what the pass came across (bbe_checked_seen), or null
+#endif
 };
+
+// Checked build: what a pass came across, for tests to see that they reach it.
+enum { kSeenContenders, kSeenListed, kSeenRest, kSeen };  // work items run on contenders alone, rollouts
+                                                          // listed to be run again, items with a rest
+#if defined(BBE_CHECKED) && BBE_CHECKED
+#define BBE_SEEN(l, what, n) \
+    do { \
+        if ((threadIdx.x & 31) == 0 && (l).seen != nullptr) atomicAdd((l).seen + (what), int(n)); \
+    } while (0)
+#else
+#define BBE_SEEN(l, what, n) ((void)0)
+#endif
 
 // An empty entry of a finishing-order hash table (no order key reaches it: keys < 2^64 - 1).
 constexpr unsigned long long kEmptyOrderKey = ~0ull;
@@ -201,6 +216,10 @@ struct bbe_batch {
     int32_t *d_queue = nullptr;        // one queue head per group
     int32_t *d_status = nullptr;       // after the queue heads
     int32_t *d_next = nullptr;         // [n_races] rollouts taken (WorkItem), after the status
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    int32_t *d_seen = nullptr;         // [kSeen] after d_next
+    bool always_contenders = false;    // look for contenders whatever that costs (bbe_checked_contenders)
+#endif
 
     bbe_launch_cfg cfg{};
     int8_t slots_by_n[BBE_MAX_COMPETITORS + 1] = {};  // layout per competitor count (0: the default)

@@ -340,8 +340,11 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         int limit = l.max_steps;  // a rollout that reaches it ends undecided
         // Finding them takes about as long as one rollout of every segment, so only where a warp runs at
         // least eight (2010 races of 10 to the sixth, 55 rollouts each: 709 us with them, 531 without).
-        if (Stage::kContenders && pass == kFirst && l.contenders && K < n_race &&
-            min(min(Rr, int64_t(l.per_lane) * (NS / n_race)), int64_t(max(l.most, w.k_count))) >= 8 * (NS / n_race)) {
+        bool worth = min(min(Rr, int64_t(l.per_lane) * (NS / n_race)), int64_t(max(l.most, w.k_count))) >= 8 * (NS / n_race);
+#if defined(BBE_CHECKED) && BBE_CHECKED
+        worth = worth || l.contenders == 2;
+#endif
+        if (Stage::kContenders && pass == kFirst && l.contenders && K < n_race && worth) {
             int H = 0;
             const unsigned front = contender_mask<DIST, LAW>(reinterpret_cast<float *>(st.ph), n_race, lane, my_d0, my_mu,
                                                              my_sg, my_P, my_kr, my_pv, my_th, L, invL, t0r, invTr, K, NS,
@@ -350,6 +353,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             if (nf >= K && (l.seg_cap > 0 ? min(NS / nf, l.seg_cap) > min(NS / n_race, l.seg_cap) : NS / nf > NS / n_race)) {
                 keep = front;
                 limit = min(limit, H);
+                BBE_SEEN(l, kSeenContenders, 1);
             }
         }
         const int n = __popc(keep);
@@ -958,6 +962,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         __syncwarp();
         const unsigned listed = st.n_redo;
         if (listed > 0u) {
+            BBE_SEEN(l, kSeenListed, listed);
             pass = kListed;
             k_begin = 0u;
             k_count = listed;
@@ -965,6 +970,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             k_begin = st.rest[0];
             k_count = st.rest[1] - k_begin;
             if (pass == kRest || k_count == 0u) break;
+            BBE_SEEN(l, kSeenRest, 1);
             pass = kRest;
         }
         }
