@@ -340,7 +340,10 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         int limit = l.max_steps;  // a rollout that reaches it ends undecided
         // Finding them takes about as long as one rollout of every segment, so only where a warp runs at
         // least eight (2010 races of 10 to the sixth, 55 rollouts each: 709 us with them, 531 without).
-        bool worth = min(min(Rr, int64_t(l.per_lane) * (NS / n_race)), int64_t(max(l.most, w.k_count))) >= 8 * (NS / n_race);
+        // Rollouts at a time: those of the item, or with tickets as many as the segments can share.
+        const int64_t at_a_time =
+            l.next != nullptr ? min(min(Rr, int64_t(l.per_lane) * (NS / n_race)), int64_t(max(l.most, w.k_count))) : w.k_count;
+        bool worth = at_a_time >= 8 * (NS / n_race);
 #if defined(BBE_CHECKED) && BBE_CHECKED
         worth = worth || l.contenders == 2;
 #endif

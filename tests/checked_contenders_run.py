@@ -158,4 +158,25 @@ for name, races, rollouts, sample in (("two", 96, 48000, 2), ("five", 96, 18000,
             want, want_s, _ = oracle.batch_places(head, 2)
             same(pc[:head.n_total], want, name)
             same(ps[:sample], want_s, name)
+
+# the no-allocation entry point, by its rule
+lib.bbe_checked_noalloc_seen.argtypes = [ctypes.c_void_p]
+dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+for name, rollouts, sample in (("two", 200000, 2), ("twenty", 8000, 4), ("twenty", 1200, 8), ("previous steps", 16000, 3),
+                               ("stuck behind the leader", 16000, 1)):
+    rb = stage(name, 96, rollouts)
+    counts = torch.empty(rb.n_total, dtype=torch.int32, device="cuda")
+    steps = torch.empty(rb.n_races, dtype=torch.int64, device="cuda")
+    bbe.bbe_rollout_noalloc(rb.n_races, rb.n_total, *(dev(a) for a in (rb.race_off, rb.L, rb.rollouts, rb.d0, rb.mu, rb.sigma,
+                                                                     rb.rho, rb.P, rb.theta)),
+                            None if rb.prev0 is None else dev(rb.prev0), rb.seed, rb.dist, rb.race_id0, counts, steps)
+    seen = np.zeros(3, np.int32)
+    assert lib.bbe_checked_noalloc_seen(seen.ctypes.data) == 0
+    print(name, rollouts, "no allocation", seen)
+    assert (seen[0] > 0) == (rollouts > 1200)  # 1200 each give every warp an item or less
+    assert seen[2] > 0 or not name.startswith("stuck")
+    head = rb.slice(0, sample)
+    want, want_s, _ = oracle.batch_counts(head)
+    same(counts[:head.n_total], want, name)
+    same(steps[:sample], want_s, name)
 print("contenders reached: ok")
