@@ -224,7 +224,8 @@ __global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, i
 }
 
 // on: the stream to build the list on, any handle, 0 (the default stream) included; none: the batch's
-// own free stream, for the calls that are given no stream.  Waits for it before returning.
+// own free stream, for the calls that are given no stream.  Waits for it before returning.  The batch is
+// left as it was if the list cannot be made: a list and the mode it was made for belong together.
 bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullopt)
 {
     const int32_t n_rec = b->n_races / b->reps;  // host records, each of `reps` equal races
@@ -238,6 +239,8 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
         double cost_full, cost_rem;
     };
     std::vector<RacePlan> plans[kGroups];
+    int8_t default_slots = 2;
+    int32_t seg_cap = 0, n_items_v[kGroups] = {};
     // keep the whole list near kMaxItems items: very large batches get larger items
     int64_t total_rollouts = 0;
     for (int r = 0; r < n_rec; ++r) total_rollouts += b->h_R[r] * b->reps;
@@ -249,8 +252,8 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
     };
     auto nseg_of = [&](int r) {  // segments of a warp: floor(32 V / n) slots of n
         const int n = b->h_off[r + 1] - b->h_off[r];
-        const int fit = 32 * slots_for(n, b->cfg.slots_per_lane, b->slots_by_n, b->default_slots) / n;
-        return b->seg_cap > 0 ? std::min(fit, b->seg_cap) : fit;
+        const int fit = 32 * slots_for(n, b->cfg.slots_per_lane, b->slots_by_n, default_slots) / n;
+        return seg_cap > 0 ? std::min(fit, seg_cap) : fit;
     };
     // A batch too small to give every warp the GPU can hold (64 per SM) a work item runs fewer
     // rollouts per lane, down to one: the chunking decides which warp runs a rollout, never its
@@ -265,8 +268,6 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
         }
         return items;
     };
-    b->default_slots = 2;
-    b->seg_cap = 0;
     while (per_lane > 1 && total_rollouts < warp_slots * per_lane * 32) {
         if (items_at(per_lane) >= warp_slots) break;
         per_lane = std::max<int64_t>(1, per_lane / 2);
@@ -276,24 +277,23 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
     // then waits on fewer segments' rank repairs; a race may then take up to one item per warp
     // slot, so that each segment runs one rollout)
     if (per_lane == 1 && total_rollouts < warp_slots * 32 && items_at(1) < warp_slots) {
-        b->default_slots = 1;
+        default_slots = 1;
         race_items = warp_slots;
         for (int32_t cap = 1; cap < 32; cap *= 2) {
-            b->seg_cap = cap;
+            seg_cap = cap;
             if (items_at(1) < warp_slots) break;
-            b->seg_cap = 0;
+            seg_cap = 0;
         }
-        if (b->seg_cap == 0) race_items = kMaxItemsPerRace;
+        if (seg_cap == 0) race_items = kMaxItemsPerRace;
     }
-    b->per_lane = int32_t(per_lane);
-    b->tickets = b->default_slots == 2;
+    const bool tickets = default_slots == 2;
     // at least four turns for each warp that is resident (28 per SM): an item too long leaves the
     // others waiting at the end
-    b->most = int32_t(std::min<int64_t>(INT32_MAX, std::max<int64_t>(1, total_rollouts / (int64_t(std::max(1, b->num_sms)) * 28 * 4))));
+    const int32_t most = int32_t(std::min<int64_t>(INT32_MAX, std::max<int64_t>(1, total_rollouts / (int64_t(std::max(1, b->num_sms)) * 28 * 4))));
     size_t total = 0;
     for (int r = 0; r < n_rec; ++r) {
         const int n = b->h_off[r + 1] - b->h_off[r];
-        const int v = slots_for(n, b->cfg.slots_per_lane, b->slots_by_n, b->default_slots);
+        const int v = slots_for(n, b->cfg.slots_per_lane, b->slots_by_n, default_slots);
         const int nseg = nseg_of(r);
         const int64_t chunk = chunk_of(r, per_lane, nseg);
         const double st = est_steps(b, r);
@@ -325,11 +325,11 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
         std::stable_sort(pg.begin(), pg.end(), [](const RacePlan &x, const RacePlan &y) { return x.cost_rem > y.cost_rem; });
         for (const RacePlan &pl : pg) {
             if (pl.rem == 0) continue;
-            if (b->tickets) runs.push_back(ItemRun{pl.race * b->reps, int32_t(pl.k0), int32_t(pl.chunk), listed});
+            if (tickets) runs.push_back(ItemRun{pl.race * b->reps, int32_t(pl.k0), int32_t(pl.chunk), listed});
             else runs.push_back(ItemRun{pl.race * b->reps, int32_t(pl.k0 + pl.full * pl.chunk), int32_t(pl.rem), listed});
             listed += b->reps;
         }
-        b->n_items_v[g] = listed - before;
+        n_items_v[g] = listed - before;
     }
 
     int32_t full = 0;  // items of full chunks per race, the same for all races of a batch with such records
@@ -343,19 +343,40 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
     ItemRun *d_runs = nullptr;
     if (!on) BBE_CUDA_TRY(ensure_free_stream(b));
     const cudaStream_t upload = on ? *on : b->free_stream;
-    BBE_CUDA_TRY(pool_alloc(reinterpret_cast<void **>(&fresh), std::max<size_t>(1, size_t(listed)) * sizeof(bbe::WorkItem), upload));
-    if (!runs.empty()) {
-        BBE_CUDA_TRY(pool_alloc(reinterpret_cast<void **>(&d_runs), runs.size() * sizeof(ItemRun), upload));
-        BBE_CUDA_TRY(cudaMemcpyAsync(d_runs, runs.data(), runs.size() * sizeof(ItemRun), cudaMemcpyHostToDevice, upload));
-        expand_items<<<unsigned((listed + 255) / 256), 256, 0, upload>>>(d_runs, int32_t(runs.size()), listed, b->tickets, full,
-                                                                            full_end, fresh);
-        BBE_CUDA_TRY(cudaGetLastError());
-        BBE_CUDA_TRY(cudaFreeAsync(d_runs, upload));
+    cudaError_t e = pool_alloc(reinterpret_cast<void **>(&fresh), std::max<size_t>(1, size_t(listed)) * sizeof(bbe::WorkItem), upload);
+    if (e == cudaSuccess && !runs.empty()) {
+        e = pool_alloc(reinterpret_cast<void **>(&d_runs), runs.size() * sizeof(ItemRun), upload);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(d_runs, runs.data(), runs.size() * sizeof(ItemRun), cudaMemcpyHostToDevice, upload);
+        if (e == cudaSuccess) {
+            expand_items<<<unsigned((listed + 255) / 256), 256, 0, upload>>>(d_runs, int32_t(runs.size()), listed, tickets, full,
+                                                                                full_end, fresh);
+            e = cudaGetLastError();
+        }
+        if (d_runs) {
+            const cudaError_t f = cudaFreeAsync(d_runs, upload);
+            if (e == cudaSuccess) e = f;
+        }
     }
-    BBE_CUDA_TRY(cudaStreamSynchronize(upload));
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    if (b->fail_list) e = cudaErrorMemoryAllocation;  // bbe_checked_fail_list
+#endif
+    const cudaError_t done = cudaStreamSynchronize(upload);  // also before `runs` goes
+    if (e == cudaSuccess) e = done;
+    if (e == cudaSuccess) e = free_behind_uses(b, b->d_items);
+    if (e != cudaSuccess) {
+        if (fresh) cudaFreeAsync(fresh, upload);
+        set_error(std::string("work list: ") + cudaGetErrorString(e));
+        return BBE_ERR_CUDA;
+    }
     free_graph(b);
-    BBE_CUDA_TRY(free_behind_uses(b, b->d_items));
     b->d_items = fresh;
+    b->default_slots = default_slots;
+    b->seg_cap = seg_cap;
+    b->per_lane = int32_t(per_lane);
+    b->most = most;
+    b->tickets = tickets;
+    std::copy(n_items_v, n_items_v + kGroups, b->n_items_v);
     return BBE_OK;
 }
 
@@ -877,8 +898,11 @@ bbe_status bbe::set_first_rollouts(bbe_batch *b, const int64_t *k0)
             return BBE_ERR_RANGE;
         }
     }
-    b->h_k0.assign(k0, k0 + b->n_races);
-    return build_items(b);
+    std::vector<int64_t> before(k0, k0 + b->n_races);
+    before.swap(b->h_k0);
+    const bbe_status st = build_items(b);
+    if (st) before.swap(b->h_k0);
+    return st;
 }
 
 cudaError_t bbe::note_use(const bbe_batch *b, cudaStream_t s)
@@ -1309,11 +1333,16 @@ bbe_status bbe_batch_set_cfg(bbe_batch *b, const bbe_launch_cfg *cfg)
     bbe_status st = check_cfg(c);
     if (st) return st;
     const bool rebuild = c.rollouts_per_lane != b->cfg.rollouts_per_lane || c.slots_per_lane != b->cfg.slots_per_lane;
+    const bbe_launch_cfg before = b->cfg;
     b->cfg = c;
+    if (rebuild && (st = build_items(b))) {
+        b->cfg = before;
+        return st;
+    }
     for (int g = 0; g < kGroups; ++g)
         b->resident[g] = bbe::rollout_resident_blocks(b->dist, kSlots[g], 32 * c.warps_per_block);
     free_graph(b);
-    return rebuild ? build_items(b) : BBE_OK;
+    return BBE_OK;
 }
 
 bbe_status bbe_batch_get_cfg(const bbe_batch *b, bbe_launch_cfg *cfg)
@@ -1352,8 +1381,12 @@ bbe_status bbe_batch_set_layout(bbe_batch *b, const int32_t *slots_by_n)
         }
         tab[n] = int8_t(slots_by_n[n]);
     }
+    int8_t before[BBE_MAX_COMPETITORS + 1];
+    std::memcpy(before, b->slots_by_n, sizeof(before));
     std::memcpy(b->slots_by_n, tab, sizeof(tab));
-    return build_items(b);
+    const bbe_status st = build_items(b);
+    if (st) std::memcpy(b->slots_by_n, before, sizeof(before));
+    return st;
 }
 
 bbe_status bbe_batch_autotune(bbe_batch *b, int32_t *win_counts, double budget_ms, void *cuda_stream)
@@ -1552,6 +1585,13 @@ BBE_API bbe_status bbe_checked_contenders(bbe_batch *b, int32_t always)
 {
     b->always_contenders = always != 0;
     free_graph(b);
+    return BBE_OK;
+}
+
+// Checked build only.  fail: the batch's next work lists cannot be made (as if memory had run out).
+BBE_API bbe_status bbe_checked_fail_list(bbe_batch *b, int32_t fail)
+{
+    b->fail_list = fail != 0;
     return BBE_OK;
 }
 

@@ -219,6 +219,7 @@ struct bbe_batch {
 #if defined(BBE_CHECKED) && BBE_CHECKED
     int32_t *d_seen = nullptr;         // [kSeen] after d_next
     bool always_contenders = false;    // look for contenders whatever that costs (bbe_checked_contenders)
+    bool fail_list = false;            // work lists cannot be made (bbe_checked_fail_list)
 #endif
 
     bbe_launch_cfg cfg{};
