@@ -228,6 +228,7 @@ __global__ void expand_items(const ItemRun *__restrict__ runs, int32_t n_runs, i
 // left as it was if the list cannot be made: a list and the mode it was made for belong together.
 bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullopt)
 {
+    std::lock_guard<std::mutex> records(b->unfold_mu);
     const int32_t n_rec = b->n_races / b->reps;  // host records, each of `reps` equal races
     // Per race: full chunks of `chunk` rollouts (all of one cost) and a remainder.  The list puts
     // longer work first: full chunks race by race in descending cost per chunk, then the
@@ -242,8 +243,7 @@ bbe_status build_items(bbe_batch *b, std::optional<cudaStream_t> on = std::nullo
     int8_t default_slots = 2;
     int32_t seg_cap = 0, n_items_v[kGroups] = {};
     // keep the whole list near kMaxItems items: very large batches get larger items
-    int64_t total_rollouts = 0;
-    for (int r = 0; r < n_rec; ++r) total_rollouts += b->h_R[r] * b->reps;
+    const int64_t total_rollouts = b->total_rollouts;
     const int64_t min_chunk = (total_rollouts + kMaxItems - 1) / kMaxItems;
     int64_t race_items = kMaxItemsPerRace;  // items per race at most (lifted for very small batches)
     auto chunk_of = [&](int r, int64_t per_lane, int nseg) {
@@ -711,6 +711,7 @@ bbe_status bbe::stage_repeated(bbe_batch **out, int32_t n_rec, int32_t reps, int
         return code;
     };
     bbe_status st = check_state(b);
+    b->total_rollouts = R * b->n_races;
     Arena A;
     if (st || (st = make_arena(b, A, s))) return fail(st);
     void *d_rec = nullptr;
@@ -839,6 +840,7 @@ bbe_status bbe::stage_batch(bbe_batch **out, int32_t n_races, const int32_t *rac
         }
     }
     if ((st = check_state(b))) return fail(st);
+    b->total_rollouts = std::accumulate(b->h_R.begin(), b->h_R.end(), int64_t(0));
     std::vector<int32_t> comp_race(nt);
     for (int r = 0; r < n_races; ++r)
         for (int i = off[r]; i < off[r + 1]; ++i) comp_race[i] = r;
@@ -1562,7 +1564,7 @@ bbe_status bbe_batch_info(const bbe_batch *b, int32_t *n_races, int64_t *n_compe
     }
     if (n_races) *n_races = b->n_races;
     if (n_competitors) *n_competitors = b->n_total;
-    if (total_rollouts) *total_rollouts = std::accumulate(b->h_R.begin(), b->h_R.end(), int64_t(0)) * b->reps;
+    if (total_rollouts) *total_rollouts = b->total_rollouts;
     if (max_competitors) *max_competitors = b->max_n;
     return BBE_OK;
 }

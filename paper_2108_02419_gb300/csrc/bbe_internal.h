@@ -195,9 +195,12 @@ struct bbe_batch {
 
     // host copies (scheduling, cost estimates, range checks and sub-batches), one record per race, or
     // one per `reps` consecutive races that differ in their stream ids alone (bbe_snapshot_batch);
-    // bbe::unfold makes it one per race for whoever needs that
+    // bbe::unfold makes it one per race for whoever needs that.  It may run in one thread while another
+    // asks for something, so whoever reads the records calls it first or holds unfold_mu, and the total of
+    // the rollouts is kept apart.
     int32_t reps = 1;
     std::mutex unfold_mu;
+    int64_t total_rollouts = 0;
     std::vector<int32_t> h_off;
     std::vector<float> h_L;
     std::vector<int64_t> h_R;
