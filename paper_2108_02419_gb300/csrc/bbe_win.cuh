@@ -60,8 +60,6 @@ namespace win {
 constexpr unsigned kAll = 0xffffffffu;
 constexpr unsigned long long kNoKey = ~0ull;
 constexpr unsigned kRedo = 64;
-constexpr int kScanMost = 6;       // competitors, at most, of a race whose i+ is found by a scan
-constexpr float kScanGap = 64.0f;  // .. and their mean distance at the start
 constexpr int kPlaced = 128;           // place mode: a segment's K places are filled, at this step of the block
 constexpr unsigned kNone = ~0u;       // win mode: a segment without a finish, ..
 constexpr unsigned kCut = kNone - 1u;  // .. and one whose rollout has run its last step without one
@@ -244,9 +242,9 @@ __device__ __forceinline__ void draw_block(const uint4 &q, uint32_t a, uint32_t 
 
 // Registers per thread: 80 for two to four slots per lane (6 resident 4-warp blocks per SM); with 72
 // (7 blocks) places to the third of 512 races of 20 take 16.3 instead of 15.2 ms, win counts the same
-// (4096 races: 31.7 and 32.2).  64 for one slot per lane, the layout of the smallest calls, which gain
-// from fewer spills, not from more warps (one small race 37 us, 42 at 56).  Three and four slots per
-// lane read their parameters from shared memory.
+// (4096 races: 31.7 and 32.2).  One slot per lane: 64 for win counts, which spill nothing then (26 batches
+// forced to that layout, 200 us or more each, 7 % faster at the mean than with 56; the smallest calls
+// the same), 56 in place mode.  Three and four slots per lane read their parameters from shared memory.
 template <int V, int MODE>
 struct WinRegs {
     static constexpr int value = V == 1 ? (MODE == 0 ? 64 : 56) : 80;
@@ -265,7 +263,6 @@ template <int DIST, int V, int LAW, int MODE>
 __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(RolloutLaunch l)
 {
     constexpr bool PS = WinLean<V>::value;
-    constexpr bool kScan = MODE == 0 && V == 1;
     using Stage = WinStage<V, MODE>;
     constexpr int NS = Stage::NS, W = Stage::W;
     constexpr int ROWB = Stage::ROW * int(sizeof(float2));
@@ -373,15 +370,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             k_count = unsigned(share < Rr - k ? share : Rr - k);
         }
         const bool kept = (keep >> lane) & 1u;
-        // Few competitors close together overtake all the time.  Where the step's latency counts (one slot
-        // per lane: the smallest calls) a look at all of them each step is shorter than keeping their order:
-        // 37.0 instead of 40.8 us for one race of 5 from the start.  With two slots per lane its
-        // instructions count, five a slot and competitor (a bettor population 7.4 instead of 6.7 ms).
-        bool scan = false;
-        if constexpr (kScan) {
-            const float back = warp_min(kept ? my_d0 : INFINITY), ahead = -warp_min(kept ? -my_d0 : INFINITY);
-            scan = n <= kScanMost && ahead - back < kScanGap * float(n - 1);
-        }
         int rank = 0;  // by (d0, index)
         for (int i = 0; i < n_race; ++i) {
             const float di = __shfl_sync(kAll, my_d0, i);
@@ -471,8 +459,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             d[v] = run ? st.d0[c] : kDead;
             pv[v] = st.prev0[c];
             const int r0 = st.rank0[c];
-            if (scan) fo[v] = min(sb, NS - n) * int(sizeof(float2));  // an unused slot looks at anything
-            else fo[v] = (run && r0 + 1 < n) ? BBE_INDEX(sb + st.byrank0[r0 + 1], NS, l.status) * int(sizeof(float2)) : kSent;
+            fo[v] = (run && r0 + 1 < n) ? BBE_INDEX(sb + st.byrank0[r0 + 1], NS, l.status) * int(sizeof(float2)) : kSent;
             if (run) {
                 st.order[BBE_INDEX(rb + r0, 2 * NS + 4, l.status)] = uint8_t(slot);
                 st.at[slot] = uint8_t(rb + r0);
@@ -773,23 +760,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 *reinterpret_cast<float2 *>(posb + BO + (32 * v + lane) * 8) = make_float2(d[v], pv[v]);
             __syncwarp();
             float fd[V], fp[V];
-            if (kScan && scan) {
-                // the nearest strictly in front, the lowest slot of equals
-#pragma unroll
-                for (int v = 0; v < V; ++v) fd[v] = fp[v] = INFINITY;
-#pragma unroll
-                for (int i = 0; i < kScanMost; ++i) {
-                    if (i < n) {
-#pragma unroll
-                        for (int v = 0; v < V; ++v) {
-                            const float2 f = *reinterpret_cast<const float2 *>(posb + BO + BBE_INDEX(fo[v], kSent + 1, l.status) + i * 8);
-                            const bool nearer = f.x > d[v] && f.x < fd[v];
-                            fd[v] = nearer ? f.x : fd[v];
-                            fp[v] = nearer ? f.y : fp[v];
-                        }
-                    }
-                }
-            } else {
             bool bad = false;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -799,7 +769,6 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                 bad |= f.x <= d[v];
             }
             if (__any_sync(kAll, bad)) repair(posb + BO, fd, fp);
-            }
             // Eq. 1 (a successor at +inf is never within theta: the free branch)
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -929,7 +898,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     const int slot = 32 * v + lane, sb = base(v);
                     const unsigned knew = st.segk[sb];
                     d[v] = kDead;
-                    if (!scan) fo[v] = kSent;
+                    fo[v] = kSent;
                     if (knew < kend) {
                         const int c = slot - sb;
                         set_stream(slot, knew, c);
@@ -937,7 +906,7 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                         d[v] = st.d0[c];
                         pv[v] = st.prev0[c];
                         const int r0 = st.rank0[c];
-                        if (!scan && r0 + 1 < n) fo[v] = (sb + st.byrank0[r0 + 1]) * int(sizeof(float2));
+                        if (r0 + 1 < n) fo[v] = (sb + st.byrank0[r0 + 1]) * int(sizeof(float2));
                         const int a = 1 + 2 * sb + r0;
                         st.order[a] = uint8_t(slot);
                         st.at[slot] = uint8_t(a);
