@@ -387,9 +387,9 @@ BBE_API void bbe_destroy_batch(bbe_batch *batch);
  * allocator that another framework holds).
  *
  * It allocates nothing: no cudaMalloc, cudaFree or allocating library call.  Its work list,
- * queue head and status word live in one file-scope device array of 1,114,144 bytes (a
- * 32-byte header, BBE_NOALLOC_MAX_RACES int32 per-race item counts and BBE_NOALLOC_MAX_ITEMS
- * 16-byte work items) that every GPU which loads the library holds until the process exits.
+ * queue head and status word live in one file-scope device array of 1,245,216 bytes (a
+ * 32-byte header, BBE_NOALLOC_MAX_RACES int32 per-race item counts, BBE_NOALLOC_MAX_ITEMS
+ * 16-byte work items and 8 bytes per race for whom the rollouts advance) that every GPU which loads the library holds until the process exits.
  * The first call on a device looks up that array's device address (cudaGetSymbolAddress)
  * with the device current; make that first call before any stream capture on the device.
  *

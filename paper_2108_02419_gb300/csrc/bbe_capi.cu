@@ -391,6 +391,36 @@ bbe_status check_cfg(const bbe_launch_cfg &c)
     return BBE_OK;
 }
 
+// Whether a pass looks for the races' contenders: where each warp has eight rollouts a segment at least to run
+// (as contender_kernel has it for each race).
+bool searches_contenders(const bbe_batch *b)
+{
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    if (b->always_contenders) return true;
+#endif
+    return b->tickets && b->per_lane >= 8;
+}
+
+// Whom a pass to the K-th finisher (places: K; 1 for win counts) advances: ahead of its rollouts on `s`.
+cudaError_t enqueue_contenders(const bbe_batch *b, int32_t places, bool place_mode, cudaStream_t s)
+{
+    if (!searches_contenders(b)) return cudaSuccess;
+    bbe::ContenderLaunch l{};
+    l.b = b->dev;
+    l.found = b->d_contenders;
+    l.places = places;
+    l.seg_cap = b->seg_cap;
+    l.status = b->d_status;
+#if defined(BBE_CHECKED) && BBE_CHECKED
+    l.always = b->always_contenders;
+#endif
+    for (int n = 1; n <= BBE_MAX_COMPETITORS; ++n) {
+        const int v = slots_for(n, b->cfg.slots_per_lane, b->slots_by_n, b->default_slots);
+        l.slots_by_n[n] = uint8_t(place_mode && v > 2 ? 0 : v);  // as WinStage::kContenders
+    }
+    return bbe::launch_contenders(l, s);
+}
+
 bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *steps, int g)
 {
     bbe::RolloutLaunch l{};
@@ -403,9 +433,8 @@ bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *ste
     l.next = b->tickets ? b->d_next : nullptr;
     l.per_lane = b->per_lane;
     l.most = b->most;
-    l.contenders = b->tickets ? 1 : 0;
+    l.contenders = searches_contenders(b) ? b->d_contenders : nullptr;
 #if defined(BBE_CHECKED) && BBE_CHECKED
-    if (b->always_contenders) l.contenders = 2;
     l.seen = b->d_seen;
 #endif
     l.counts = counts;
@@ -444,6 +473,7 @@ cudaError_t enqueue_pass(const bbe_batch *b, int32_t *counts, int64_t *steps, cu
     int groups[kGroups], ng = 0;
     for (int g = kGroups - 1; g >= 0; --g)
         if (b->n_items_v[g] > 0) groups[ng++] = g;
+    if (e == cudaSuccess) e = enqueue_contenders(b, 1, false, s);
     if (e != cudaSuccess || ng == 0) return e;
     if (ng > 1 && side) {
         e = cudaEventRecord(b->ev_fork, s);
@@ -578,6 +608,7 @@ bbe_status make_arena(bbe_batch *b, Arena &A, cudaStream_t s)
     add((n_races + 1) * 4); add(n_races * 4); add(n_races * 8); add(nt * 4); add(n_races * 4);
     for (int i = 0; i < 7; ++i) add(nt * 4);
     add((kGroups + 1 + n_races + bbe::kSeen) * 4);
+    add(n_races * sizeof(bbe::Contenders));
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e == cudaSuccess) e = pool_alloc(&b->arena, bytes, s);
@@ -596,6 +627,7 @@ bbe_status make_arena(bbe_batch *b, Arena &A, cudaStream_t s)
     b->d_queue = carve<int32_t>(p, kGroups + 1 + n_races + bbe::kSeen);
     b->d_status = b->d_queue + kGroups;
     b->d_next = b->d_status + 1;
+    b->d_contenders = carve<bbe::Contenders>(p, n_races);
 #if defined(BBE_CHECKED) && BBE_CHECKED
     b->d_seen = b->d_next + n_races;
 #endif
@@ -981,6 +1013,7 @@ bbe_status run_place_mode(bbe_batch *b, int32_t places, int32_t *place_counts, i
         BBE_CUDA_TRY(cudaMemsetAsync(place_counts, 0, size_t(b->n_total) * size_t(places) * sizeof(int32_t), s));
     if (steps_total) BBE_CUDA_TRY(cudaMemsetAsync(steps_total, 0, size_t(b->n_races) * sizeof(int64_t), s));
     BBE_CUDA_TRY(reset_queue(b, s));
+    BBE_CUDA_TRY(enqueue_contenders(b, places, true, s));
     for (int g = kGroups - 1; g >= 0; --g) {
         if (b->n_items_v[g] == 0) continue;
         bbe::RolloutLaunch l = make_launch(b, place_counts, steps_total, g);

@@ -55,6 +55,13 @@ struct WorkItem {
     int32_t pad;
 };
 
+// The competitors of a race that the rollout kernel advances (a bit each), and the steps for which a rollout of
+// these alone is one of the whole race (INT_MAX with all of them).
+struct Contenders {
+    uint32_t keep;
+    int32_t horizon;
+};
+
 struct RolloutLaunch {
     DevBatch b;
     const WorkItem *items;
@@ -63,7 +70,7 @@ struct RolloutLaunch {
     int32_t *next;            // [n_races] tickets' worth of rollouts taken, zeroed before each launch; null: none
     int32_t per_lane;         // with next: rollouts per segment that a warp takes at a time, ..
     int32_t most;             // .. and in all, unless one ticket is worth more
-    int32_t contenders;       // advance only the competitors that can matter (contender_mask)
+    const Contenders *contenders;  // [n_races] who is advanced (bbe_contenders.cu); null: everybody
     int32_t *counts;          // [n_total]
     unsigned long long *steps;  // [n_races] or null
     int32_t *status;          // device status bits
@@ -81,6 +88,17 @@ struct RolloutLaunch {
 #if defined(BBE_CHECKED) && BBE_CHECKED
     int32_t *seen;           // [kSeen] what the pass came across (bbe_checked_seen), or null
 #endif
+};
+
+// The search for the races' contenders, to the K-th place (places; 1: win counts).
+struct ContenderLaunch {
+    DevBatch b;
+    Contenders *found;  // [n_races]
+    int32_t places;
+    int32_t seg_cap;    // as RolloutLaunch's
+    int32_t *status;
+    bool always;        // checked build: search whatever it costs
+    uint8_t slots_by_n[BBE_MAX_COMPETITORS + 1];  // slots per lane of a race of n; 0: everybody is advanced
 };
 
 // Checked build: what a pass came across, for tests to see that they reach it.
@@ -175,6 +193,8 @@ int place_resident_blocks(int dist, int slots_per_lane, int block, int place_cel
 cudaError_t launch_place_probs(const DevBatch &b, int places, const int32_t *counts, int top, float *probs,
                                cudaStream_t stream);
 
+cudaError_t launch_contenders(const ContenderLaunch &l, cudaStream_t stream);
+
 void set_error(const std::string &msg);
 
 }  // namespace bbe
@@ -219,6 +239,7 @@ struct bbe_batch {
     int32_t *d_queue = nullptr;        // one queue head per group
     int32_t *d_status = nullptr;       // after the queue heads
     int32_t *d_next = nullptr;         // [n_races] rollouts taken (WorkItem), after the status
+    bbe::Contenders *d_contenders = nullptr;  // [n_races] who is advanced, found anew by each pass
 #if defined(BBE_CHECKED) && BBE_CHECKED
     int32_t *d_seen = nullptr;         // [kSeen] after d_next
     bool always_contenders = false;    // look for contenders whatever that costs (bbe_checked_contenders)

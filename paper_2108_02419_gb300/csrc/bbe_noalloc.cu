@@ -43,6 +43,7 @@ struct NoallocScratch {
     NoallocHeader h;
     int32_t race_items[kMaxRaces];   // per-race item counts, then offsets
     bbe::WorkItem items[kMaxItems];  // the work list, race by race
+    bbe::Contenders contenders[kMaxRaces];
 };
 
 // The only memory this entry point uses besides the caller's arrays.  Host code must not
@@ -281,11 +282,19 @@ extern "C" BBE_API bbe_status bbe_rollout_noalloc(int32_t n_races, int32_t n_com
 #endif
         l.block = block;
         l.grid = sms * std::max(1, std::min(16, bbe::rollout_resident_blocks(int(dist), kSlots, block)));
-        // Contenders where the items outnumber the resident warps: 512 races of 20, 10^4 rollouts each 4.7
-        // instead of 11.6 ms, 64 of them (1.6 items a warp) 1.2 instead of 2.0.  With an item a warp or less
-        // the slowest race decides, and that is one where everybody matters, which pays for the search
-        // without a gain: 1000 races of 10, 60 rollouts each 0.58 instead of 0.50 ms, 200 each 1.46 and 1.47.
-        l.contenders = l.n_items > l.grid * (block / 32) ? 1 : 0;
+        // Contenders where the items outnumber the resident warps: 512 races of 20, 10^4 rollouts each 3.8
+        // instead of 11.6 ms, 64 of them (1.6 items a warp) 1.1 instead of 2.0.  With an item a warp or less
+        // the slowest race decides, and that is one where everybody matters.
+        if (l.n_items > l.grid * (block / 32)) {
+            bbe::ContenderLaunch c{};
+            c.b = b;
+            c.found = sc->contenders;
+            c.places = 1;
+            c.status = &sc->h.status;
+            for (int n = 1; n <= BBE_MAX_COMPETITORS; ++n) c.slots_by_n[n] = kSlots;
+            NA_TRY(bbe::launch_contenders(c, s));
+            l.contenders = sc->contenders;
+        }
         l.grid = std::max(1, std::min(l.grid, (l.n_items + block / 32 - 1) / (block / 32)));  // no idle warps
         bbe::fill_round_keys(l);
         NA_TRY(bbe::launch_rollout(l, kSlots, s));

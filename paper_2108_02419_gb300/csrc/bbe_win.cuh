@@ -25,7 +25,7 @@
 // its rollouts run out.
 //
 // Who is advanced.  Only the competitors that can matter to the first finish, or the first K, are
-// (contender_mask); they take the slots, so a warp has room for more segments.  A work item is a
+// (bbe_contenders.cu); they take the slots, so a warp has room for more segments.  A work item is a
 // ticket for some of a race's rollouts, and the warp takes as many as its segments can share.
 //
 // Finishing.  A rollout that ends waits for the block's end in any case, and what its slots do until
@@ -100,125 +100,6 @@ struct WinStage {
     uint8_t rank0[32], byrank0[32];     // start rank of competitor c; competitor at start rank r
     uint8_t comp[32];                   // the race's index of competitor c (its stream and its count)
 };
-
-__device__ __forceinline__ float warp_min(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(kAll, v, o));
-    return v;
-}
-
-__device__ __forceinline__ float warp_max(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kAll, v, o));
-    return v;
-}
-
-// The contenders of a race.  The first K finishers are decided among the competitors near the front, and
-// Eq. 1 passes influence from front to back only, so a competitor that is certain to stay short of the
-// line until a rollout ends cannot change its first K places, nor when they are filled.
-// contender_mask returns the competitors that are not ruled out so: in every rollout that ends within
-// H steps (H is set here), a rollout of these alone, each on its own stream, has the same first K
-// finishers and the same number of steps.
-//
-// The bound, for any draws.  E_i(t) bounds the position after t steps of every competitor that starts at or
-// behind rank i (ranks by start position) and of everyone that one of them has affected (the affected
-// were behind it, so the bound holds for them from there on).  A free step is at most F = max R P (mu +
-// z_max sigma), the largest over the competitors (the generator's |z| is bounded: u1 >= 2^-24 gives a
-// radius of at most 5.7681; sqrt(3) and 1 for the other two distributions) and at least the previous
-// steps given.  A blocked step is R min(own previous step, that of the competitor in front), so with lambda
-// the largest R where it happens,
-//   S_c(t) > lambda^k F  =>  S(t-1) > lambda^(k-1) F for c and for the one in front of it, within theta,
-// and the foremost of those who have S(t-i) > lambda^(k-i) F has one in front that is not among them:
-// k levels take k members whose R can exceed 1, each within n theta of another at some of the last k
-// steps.  A member that was there i steps ago has fallen back since by at most i steps' difference
-// between the largest step and F, by less than M in all.  So if j is the rearmost member, c is at most M
-// ahead of E_j, the others rank above j and started behind E_j + M + n theta, and those are counted
-// (k_j, lambda_j):
-//   V_j = F lambda_j^k_j,   E_i(t+1) = max over j <= i of min(E_j(t) + M, E_i(t)) + V_j.
-// M for step t follows from the levels of the step before, which a step exceeds by one at most.  Rounding is
-// covered by the factors and the margins.  A competitor is ruled out when its E stays short of the
-// line for H steps.  (With one bound for everybody's advance, the closest groups anywhere on the
-// track count against all: 10 contenders of 20 at the mean in the uniform batch, 4.8 with this one.)
-//
-// H is an estimate of the K-th finish with a margin of three standard deviations; the few rollouts
-// that are still running after H steps are run again with everybody.
-// x: 3 n floats of scratch; slots: of the warp.  Called by the whole warp; lane c < n holds competitor c.
-template <int DIST, int LAW>
-__device__ __forceinline__ unsigned contender_mask(float *x, int n, int lane, float d, float mu, float sigma, float P,
-                                                   float kr, float prev, float theta, float L, float invL, float t0,
-                                                   float invT, int K, int slots, int &H)
-{
-    const bool on = lane < n;
-    const unsigned everybody = kAll >> (32 - n);
-    constexpr float zmax = DIST == BBE_DIST_NORMAL ? 5.769f : (DIST == BBE_DIST_UNIFORM ? 1.7321f : 1.0f);
-    // expected finish at the R of the middle of the way, and the horizon: the K-th least with its margin
-    float T = (L - d) / (mu * P);
-    T /= 1.0f + (LAW == BBE_LAW_TIME ? kr * (fminf((t0 + 0.5f * T) * invT, 1.0f) - 0.5f) : 0.5f * kr * d * invL);
-    const float h = on ? T + 3.0f * sigma * sqrtf(T) / mu + 1.0f : INFINITY;
-    int rank = 0, hrank = 0;  // by (start position, index) and by (horizon, index)
-    for (int i = 0; i < n; ++i) {
-        const float di = __shfl_sync(kAll, d, i), hi = __shfl_sync(kAll, h, i);
-        rank += di < d || (di == d && i < lane) ? 1 : 0;
-        hrank += hi < h || (hi == h && i < lane) ? 1 : 0;
-    }
-    const float hk = warp_max(on && hrank < K ? h : 0.0f);
-    const float margin = float(n) * warp_max(on ? theta : 0.0f);
-    if (!(hk < 1e6f) || !(margin < L)) return everybody;
-    H = int(hk) + 1;
-    // R is linear in the position or the time: largest at an end of its range
-    const float lo = LAW == BBE_LAW_TIME ? fminf(t0 * invT, 1.0f) : d * invL;
-    const float end = LAW == BBE_LAW_TIME ? fminf((t0 + float(H)) * invT, 1.0f) : (L + margin) * invL;
-    const float Rlo = 1.0f + kr * (lo - 0.5f);
-    const float R = 1.00001f * fmaxf(Rlo, 1.0f + kr * (end - 0.5f));
-    const float F = 1.0001f * fmaxf(warp_max(on ? fmaxf(prev, R * P * (mu + zmax * sigma)) : 0.0f), kStepFloor);
-    const float goal = 0.9999f * L;
-    // not even at the free pace would there be room for more segments
-    if (slots / max(1, __popc(__ballot_sync(kAll, on && !(goal - float(H) * F > d)))) <= slots / n) return everybody;
-    const float lambda = 1.00001f * fmaxf(warp_max(on ? R : 0.0f), 1.0f);  // anywhere
-    // from here on lane i holds rank i
-    if (on) {
-        x[rank] = d;
-        x[n + rank] = kr;
-        x[2 * n + rank] = Rlo;
-    }
-    __syncwarp();
-    float E = on ? x[lane] : INFINITY, M = margin;
-    float rise = 0.0f, Rmax = 1.0f;  // of the ranks lane .. next - 1: the largest kr, and R at the range's start
-    int next = lane, early = 0, late = 0;  // those whose R exceeds 1 there, and those later on only
-    for (int t = 0; t < H;) {
-        while (next < n && x[next] <= E + M + margin) {
-            const float k1 = x[n + next], r1 = x[2 * n + next];
-            Rmax = fmaxf(Rmax, r1);
-            if (r1 > 0.9999f) ++early;
-            else if (k1 > 0.0f) ++late;
-            rise = fmaxf(rise, k1);
-            ++next;
-        }
-        const float now = LAW == BBE_LAW_TIME ? fminf((t0 + float(t)) * invT, 1.0f) : fminf((E + M + margin) * invL, end);
-        const int k = early + (now > 0.4999f ? late : 0);
-        const float lam = 1.00001f * fmaxf(Rmax, 1.0f + rise * (now - 0.5f));
-        const float V = on ? 1.0001f * F * powf(lam, float(k)) : 0.0f;
-        float En = E + V;
-        for (int j = 0; j + 1 < n; ++j) {
-            const float Ej = __shfl_sync(kAll, E, j), Vj = __shfl_sync(kAll, V, j);
-            if (j < lane) En = fmaxf(En, fminf(Ej + M, E) + Vj);
-        }
-        E = En;
-        if (__shfl_sync(kAll, E, 0) >= goal) {
-            __syncwarp();
-            return everybody;
-        }
-        const int km = __reduce_max_sync(kAll, on ? k : 0);
-        M = fmaxf(M, margin + float(km) * F * (1.0002f * powf(lambda, float(km)) - 1.0f));
-        ++t;
-    }
-    const float bound = __shfl_sync(kAll, E, rank & 31);
-    const bool out = on && !(bound >= goal);
-    __syncwarp();
-    return everybody & ~__ballot_sync(kAll, out);
-}
 
 template <int DIST>
 __device__ __forceinline__ void draw_block(const uint4 &q, uint32_t a, uint32_t blk, const uint32_t (&rkey)[20],
@@ -331,29 +212,15 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
             my_kr = __fmul_rn(kKappa, __fsub_rn(__fmul_rn(2.0f, b.rho[ci]), 1.0f));
             my_pv = b.prev0 ? b.prev0[ci] : __fmul_rn(my_mu, my_P);
         }
-        // the n competitors advanced, in the race's order: all of them, or the contenders where
-        // that makes room for more segments
+        // the n competitors advanced, in the race's order: all of them, or the contenders
         unsigned keep = kAll >> (32 - n_race);
         int limit = l.max_steps;  // a rollout that reaches it ends undecided
-        // Finding them takes about as long as one rollout of every segment, so only where a warp runs at
-        // least eight (2010 races of 10 to the sixth, 55 rollouts each: 709 us with them, 531 without).
-        // Rollouts at a time: those of the item, or with tickets as many as the segments can share.
-        const int64_t at_a_time =
-            l.next != nullptr ? min(min(Rr, int64_t(l.per_lane) * (NS / n_race)), int64_t(max(l.most, w.k_count))) : w.k_count;
-        bool worth = at_a_time >= 8 * (NS / n_race);
-#if defined(BBE_CHECKED) && BBE_CHECKED
-        worth = worth || l.contenders == 2;
-#endif
-        if (Stage::kContenders && pass == kFirst && l.contenders && K < n_race && worth) {
-            int H = 0;
-            const unsigned front = contender_mask<DIST, LAW>(reinterpret_cast<float *>(st.ph), n_race, lane, my_d0, my_mu,
-                                                             my_sg, my_P, my_kr, my_pv, my_th, L, invL, t0r, invTr, K, NS,
-                                                             H);
-            const int nf = __popc(front);
-            if (nf >= K && (l.seg_cap > 0 ? min(NS / nf, l.seg_cap) > min(NS / n_race, l.seg_cap) : NS / nf > NS / n_race)) {
-                keep = front;
-                limit = min(limit, H);
-                BBE_SEEN(l, kSeenContenders, 1);
+        if constexpr (Stage::kContenders) {
+            if (pass == kFirst && l.contenders != nullptr) {
+                const Contenders who = l.contenders[r];
+                if (who.keep != keep) BBE_SEEN(l, kSeenContenders, 1);
+                keep = who.keep;
+                limit = min(limit, who.horizon);
             }
         }
         const int n = __popc(keep);
