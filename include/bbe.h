@@ -129,7 +129,8 @@ typedef struct {
  *               split into pieces reproduces the counts of the whole.
  *   cuda_stream stream for the staging copies; the call synchronises it before returning.
  * Every array may live in host or device memory and is read in the stream's order (after the work
- * enqueued before the call, host memory that this work writes included); the library keeps its own device copy, so the caller may free them after the call.
+ * enqueued before the call, host memory that this work writes included); the library keeps its
+ * own device copy, so the caller may free them after the call.
  * Errors: BBE_ERR_ARG, BBE_ERR_UNSUPPORTED, BBE_ERR_FINISHED, BBE_ERR_CUDA. */
 BBE_API bbe_status bbe_race_init(bbe_batch **out, int32_t n_races, const int32_t *race_off, const float *track_len,
                          const int64_t *rollouts, const float *pos, const float *mu, const float *sigma,

@@ -58,8 +58,9 @@ __device__ __forceinline__ float warp_max(float v)
 // line for H steps.  (With one bound for everybody's advance, the closest groups anywhere on the
 // track count against all: 10 contenders of 20 at the mean in the uniform batch, 4.8 with this one.)
 //
-// H is an estimate of the K-th finish with a margin of three standard deviations; the few rollouts
-// that are still running after H steps are run again with everybody.
+// H is an estimate of the K-th finish with a margin of three standard deviations (two and four: within 2 % for
+// 4096 spread races of 20, 10^4 uneven ones and places); the few rollouts that are still running after
+// H steps are run again with everybody.
 // x: 3 n floats of scratch; most: contenders, at most, that leave room for more segments (else everybody is
 // returned, as soon as that is certain: a bound grows by its own advance of this step at least in every
 // later one, as its members and their R only grow).  Called by the whole warp; lane c < n holds competitor c.

@@ -79,7 +79,8 @@ struct WinStage {
     float d0[32], prev0[32];            // per competitor: start state of every rollout
     uint4 ph[NS];                       // per slot: the current rollout's Philox constants (StreamWords)
     unsigned segk[NS];                  // by segment base: its rollout
-    // rollouts to run again with everybody: a warp takes no more new ones once kRedo are listed
+    // rollouts to run again with everybody: a warp takes no more new ones once kRedo are listed (16 or 256: the same
+    // times, few rollouts are listed)
     static constexpr bool kContenders = MODE == 0 || V <= 2;
     unsigned redo[kContenders ? kRedo + NS : 1];
     unsigned n_redo, rest[2];           // how many; first and end of those not begun for their number
@@ -340,6 +341,9 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
         // first later rank strictly in front.  (A count of every slot's rank, over all of its segment, took
         // 727 instead of 346 us where chains of overtakes are the rule: 116 bunched races of 30 to the sixth
         // place, 170 rollouts each; 700 of 13 14.45 instead of 14.16 ms.)  pb is the step's row.
+        // In a pass a slot whose turn it is not reads its successor's entry while the pair behind it may be
+        // swapping: it finds one or the other, which only decides whether there is another pass, and there is
+        // one wherever somebody swapped.  Entries that count are read in passes that write none of them.
         auto full_sort = [&](const char *pb, float (&fd)[V], float (&fp)[V]) {
             const float2 *row = reinterpret_cast<const float2 *>(pb);
             __syncwarp();
@@ -677,9 +681,9 @@ __global__ void __maxnreg__((WinRegs<V, MODE>::value)) win_rollout_kernel(Rollou
                     draw_block<DIST>(st.ph[32 * v + lane], PS ? st.pha[kra[v] - st.kr] : pha[v], blk[v], l.round_key, z[v]);
             };
             if constexpr (MODE == 0) {
-                // two copies of the step, run twice (the second time with the block's other two normals): with four, the steps and their repairs overflow the instruction cache where
-                // overtakes are frequent (700 bunched races of 13: 15.3 instead of 14.6 ms; spread races
-                // without overtakes lose 1 to 2 %)
+                // two copies of the step, run twice (the second time with the block's other two normals): with
+                // four, the steps and their repairs overflow the instruction cache where overtakes are frequent
+                // (700 bunched races of 13: 15.3 instead of 14.6 ms; spread races without overtakes lose 1 to 2 %)
 #pragma unroll 1
                 for (j0 = 0; j0 < W; j0 += 2) {
                     if (j0 == 0) {
