@@ -122,9 +122,9 @@ __device__ __forceinline__ void draw_block(const uint4 &q, uint32_t a, uint32_t 
     }
 }
 
-// Registers per thread: 80 for two to four slots per lane (6 resident 4-warp blocks per SM); with 72
-// (7 blocks) places to the third of 512 races of 20 take 16.3 instead of 15.2 ms, win counts the same
-// (4096 races: 31.7 and 32.2).  One slot per lane: 64 for win counts, which spill nothing then (26 batches
+// Registers per thread: 80 for two to four slots per lane (6 resident 4-warp blocks per SM); with 72 and
+// 7 blocks it is the same (4096 races of 20 24.6 and 24.4 ms, places to the third of 512 12.6 and 12.5, full
+// orders of 96 19.1 both).  One slot per lane: 64 for win counts, which spill nothing then (26 batches
 // forced to that layout, 200 us or more each, 7 % faster at the mean than with 56; the smallest calls
 // the same), 56 in place mode.  Three and four slots per lane read their parameters from shared memory.
 template <int V, int MODE>
