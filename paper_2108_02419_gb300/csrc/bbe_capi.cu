@@ -392,19 +392,20 @@ bbe_status check_cfg(const bbe_launch_cfg &c)
 }
 
 // Whether a pass looks for the races' contenders: where each warp has eight rollouts a segment at least to run
-// (as contender_kernel has it for each race).
-bool searches_contenders(const bbe_batch *b)
+// (as contender_kernel has it for each race) and to the K-th finisher (places: K; 1 for win counts) of more.
+bool searches_contenders(const bbe_batch *b, int32_t places)
 {
+    if (places >= b->max_n) return false;
 #if defined(BBE_CHECKED) && BBE_CHECKED
     if (b->always_contenders) return true;
 #endif
     return b->tickets && b->per_lane >= 8;
 }
 
-// Whom a pass to the K-th finisher (places: K; 1 for win counts) advances: ahead of its rollouts on `s`.
+// Whom a pass advances, ahead of its rollouts on `s`.
 cudaError_t enqueue_contenders(const bbe_batch *b, int32_t places, bool place_mode, cudaStream_t s)
 {
-    if (!searches_contenders(b)) return cudaSuccess;
+    if (!searches_contenders(b, places)) return cudaSuccess;
     bbe::ContenderLaunch l{};
     l.b = b->dev;
     l.found = b->d_contenders;
@@ -421,7 +422,7 @@ cudaError_t enqueue_contenders(const bbe_batch *b, int32_t places, bool place_mo
     return bbe::launch_contenders(l, s);
 }
 
-bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *steps, int g)
+bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *steps, int g, int32_t places = 1)
 {
     bbe::RolloutLaunch l{};
     l.b = b->dev;
@@ -433,7 +434,7 @@ bbe::RolloutLaunch make_launch(const bbe_batch *b, int32_t *counts, int64_t *ste
     l.next = b->tickets ? b->d_next : nullptr;
     l.per_lane = b->per_lane;
     l.most = b->most;
-    l.contenders = searches_contenders(b) ? b->d_contenders : nullptr;
+    l.contenders = searches_contenders(b, places) ? b->d_contenders : nullptr;
 #if defined(BBE_CHECKED) && BBE_CHECKED
     l.seen = b->d_seen;
 #endif
@@ -1016,7 +1017,7 @@ bbe_status run_place_mode(bbe_batch *b, int32_t places, int32_t *place_counts, i
     BBE_CUDA_TRY(enqueue_contenders(b, places, true, s));
     for (int g = kGroups - 1; g >= 0; --g) {
         if (b->n_items_v[g] == 0) continue;
-        bbe::RolloutLaunch l = make_launch(b, place_counts, steps_total, g);
+        bbe::RolloutLaunch l = make_launch(b, place_counts, steps_total, g, places);
         l.places = places;
         l.orders = orders;
         l.order_off = orders ? b->d_order_off : nullptr;
